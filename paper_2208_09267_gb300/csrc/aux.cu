@@ -12,7 +12,7 @@ cudaError_t launch_step_fast_d1q3(const LatticeDev *, int, bool, int, int, const
 cudaError_t launch_step_fast_d2q9(const LatticeDev *, int, bool, int, int, const StepLaunch &, cudaStream_t);
 cudaError_t launch_step_fast_d3q19(const LatticeDev *, int, bool, int, int, const StepLaunch &, cudaStream_t);
 cudaError_t launch_step_fast_d3q27(const LatticeDev *, int, bool, int, int, const StepLaunch &, cudaStream_t);
-cudaError_t launch_step_exact(int lattice, const LatticeDev *L_dev, bool odd, int red, int k,
+cudaError_t launch_step_exact(const LatticeDev &h, const LatticeDev *L_dev, bool odd, int red, int k,
                               const StepLaunch &ls, cudaStream_t s);
 cudaError_t launch_step_row_d2q9(const LatticeDev *, int, bool, int, int, const StepLaunch &, cudaStream_t);
 cudaError_t launch_step_row_d3q19(const LatticeDev *, int, bool, int, int, const StepLaunch &, cudaStream_t);
@@ -54,10 +54,29 @@ StepLaunch make_launch(int nx, int ny, int nz, int bx, int by) {
   return ls;
 }
 
+// The FP64 step is bound by the FP64 pipe of each SM, so the blocks are made
+// small enough to deal the warps evenly: the largest of 256, 128, 64 threads
+// that still gives 8 blocks per SM, else one warp per block.  64 x 64 cells
+// are 128 warps, one SM each: 10.0 us a step (18.7 as 16 blocks of 256
+// threads, 10.8 as 32 of 128); 256 x 256: 32.6 us (35.9 in blocks of 128 or
+// more); 48^3 and 64^3 do not depend on it.
+StepLaunch make_launch_exact(int nx, int ny, int nz, int bx, int by) {
+  StepLaunch ls = make_launch(nx, ny, nz, bx, by);
+  const long long cells = (long long)nx * ny * nz;
+  if (bx <= 0 || by <= 0) {
+    int t = 256;
+    while (t > 32 && (cells + t - 1) / t < 8LL * 152) t /= 2;
+    ls.block = dim3(t, 1, 1);
+  }
+  ls.block_threads = (int)(ls.block.x * ls.block.y);
+  ls.grid = dim3((unsigned)((cells + ls.block_threads - 1) / ls.block_threads), 1, 1);
+  return ls;
+}
+
 cudaError_t launch_step(const LatticeDev &h, const LatticeDev *L_dev, long long n_host, int k, int red,
                         const StepLaunch &ls, cudaStream_t s) {
   const bool odd = ((n_host + k) & 1) != 0;
-  if (h.storage == 0) return launch_step_exact(h.lattice, L_dev, odd, red, k, ls, s);
+  if (h.storage == 0) return launch_step_exact(h, L_dev, odd, red, k, ls, s);
   if (ls.row) {
     // bit 1: this step decodes with the previous phi's shift (set_epsilon
     // since the last step); the row kernel is instantiated for both cases

@@ -97,6 +97,8 @@ int plan_row_kernel(int lattice, int storage, int nx, int nxp, int ny, int nz, u
 
 // Default/chosen block shape -> launch geometry for a lattice.
 StepLaunch make_launch(int nx, int ny, int nz, int bx, int by);
+// The FP64 step's: cells in linear order, bx*by threads per block.
+StepLaunch make_launch_exact(int nx, int ny, int nz, int bx, int by);
 
 // Launch one fused step (parity from n_host) of a single lattice, reading
 // the descriptor at L_dev.  `k` is added to the device-side time counter

@@ -186,7 +186,9 @@ extern "C" size_t lbm_vanse_device_bytes(const lbm_vanse_params *p, int with_dep
   if (p->storage != LBM_FP64) b += 2 * (size_t)N * 2;       // shift double buffer
   if (with_deps) b += 2 * (size_t)N * fe;                   // d_t phi double buffer
   if (with_force_field) b += 2 * 3 * (size_t)N * fe;
-  const lbm::StepLaunch ls = lbm::make_launch(p->nx, p->ny, p->nz, p->block_x, p->block_y);
+  const lbm::StepLaunch ls = p->storage == LBM_FP64
+                                 ? lbm::make_launch_exact(p->nx, p->ny, p->nz, p->block_x, p->block_y)
+                                 : lbm::make_launch(p->nx, p->ny, p->nz, p->block_x, p->block_y);
   size_t nb = (size_t)ls.grid.x * ls.grid.y * ls.grid.z;
   if (nb < kRowGridBound) nb = kRowGridBound;
   b += nb * lbm::kRedWidth * sizeof(double);
@@ -319,7 +321,8 @@ extern "C" int lbm_vanse_create(const lbm_vanse_params *p, lbm_vanse_t *out) {
     m.scale = m.inv_scale = 1.0f;
   }
 
-  h->ls = lbm::make_launch(p->nx, p->ny, p->nz, p->block_x, p->block_y);
+  h->ls = p->storage == LBM_FP64 ? lbm::make_launch_exact(p->nx, p->ny, p->nz, p->block_x, p->block_y)
+                                 : lbm::make_launch(p->nx, p->ny, p->nz, p->block_x, p->block_y);
   h->nblocks = (int)(h->ls.grid.x * h->ls.grid.y * h->ls.grid.z);
   h->ls.row_consumers = p->row_consumers;
   h->ls.row_stages = p->row_stages;

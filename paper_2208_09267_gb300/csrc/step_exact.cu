@@ -81,9 +81,11 @@ struct MacroD {
   double M0, J[3], I, rho, F[3], u[3];
 };
 
-template <class LAT>
+// phi at time n of the FP64 fields (F64) or of the FP32 fields of the other
+// storages, in double.
+template <bool F64>
 __device__ __forceinline__ double eps_at(const LatticeDev &L, long long m, double dn) {
-  if (L.storage == 0) {
+  if (F64) {
     const double *e = static_cast<const double *>(L.eps);
     if (L.has_deps) return e[m] + dn * static_cast<const double *>(L.deps)[m];
     return e[m];
@@ -93,10 +95,10 @@ __device__ __forceinline__ double eps_at(const LatticeDev &L, long long m, doubl
   return (double)e[m];
 }
 
-template <class LAT>
+template <bool F64>
 __device__ __forceinline__ double force_at(const LatticeDev &L, int a, long long k, double dnf) {
   const long long off = (long long)a * L.ncell + k;
-  if (L.storage == 0) {
+  if (F64) {
     double fa = static_cast<const double *>(L.force)[off];
     if (L.has_dforce) fa = fa + dnf * static_cast<const double *>(L.dforce)[off];
     return fa;
@@ -106,27 +108,68 @@ __device__ __forceinline__ double force_at(const LatticeDev &L, int a, long long
   return fa;
 }
 
+// What bounds the FP64 kernels: the FP64 pipe takes 64 clocks for a warp
+// instruction on each quarter of an SM, 19 with all four busy (measured; the
+// lanes in use do not matter), a 64th of the FP32 rate, so every operation
+// below counts and loads do not.  The operations are
+// those of the canonical order with the ones that cannot change a result
+// left out: terms with a zero velocity component (x + 0 y = x for finite
+// y), products by +-1 and +-1/2 (exact, so they move freely; J + F/2 is one
+// FMA), and what a population shares with its opposite (c u and c F change
+// sign exactly, (4.5 cu) cu and (9 cu) cF do not).  About 240 operations per
+// D2Q9 cell, 430 D3Q19, 600 D3Q27: a 48^3 D3Q27 step 138 us (before 240), a
+// 64 x 64 D2Q9 step 9.6 us (26, most of it from the smaller blocks of
+// make_launch_exact).
+
+// sum over the velocities of one set of c_ia v_a, terms in ascending a
 template <class LAT>
-__device__ __forceinline__ void macro_exact(const LatticeDev &L, long long n, const Coords &C,
-                                            const double *f, MacroD &m) {
-  constexpr int Q = LAT::Q, D = LAT::D;
-  m.M0 = 0.0;
+__device__ __forceinline__ double dot_c(int i, const double *v) {
+  double s = 0.0;
+  bool any = false;
 #pragma unroll
-  for (int i = 0; i < Q; ++i) m.M0 = m.M0 + f[i];
+  for (int a = 0; a < LAT::D; ++a) {
+    if (LAT::c(i, a) == 0) continue;
+    const double t = LAT::c(i, a) > 0 ? v[a] : -v[a];
+    s = any ? s + t : t;
+    any = true;
+  }
+  return s;
+}
+
+// M0 and J in ascending i
+template <class LAT>
+__device__ __forceinline__ void sums_exact(const double *f, MacroD &m) {
+  constexpr int Q = LAT::Q, D = LAT::D;
+  m.M0 = f[0];
+#pragma unroll
+  for (int i = 1; i < Q; ++i) m.M0 = m.M0 + f[i];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     m.J[a] = 0.0;
+    if (a >= D) continue;
+    bool any = false;
 #pragma unroll
-    for (int i = 0; i < Q; ++i) m.J[a] = m.J[a] + (double)LAT::c(i, a) * f[i];
+    for (int i = 1; i < Q; ++i) {
+      if (LAT::c(i, a) == 0) continue;
+      const double t = LAT::c(i, a) > 0 ? f[i] : -f[i];
+      m.J[a] = any ? m.J[a] + t : t;
+      any = true;
+    }
   }
+}
+
+// rho~, F and u from M0 and J; DRAG: the lattice may carry the drag law
+template <class LAT, bool F64, bool DRAG>
+__device__ __forceinline__ void macro_from_sums(const LatticeDev &L, long long n, const Coords &C, MacroD &m) {
+  constexpr int D = LAT::D;
   const double dn = (double)(n - L.n_eps);
-  const double e_c = eps_at<LAT>(L, C.at(0, 0, 0), dn);
+  const double e_c = eps_at<F64>(L, C.at(0, 0, 0), dn);
   double e_p[3], e_m[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     if (a < D) {
-      e_p[a] = eps_at<LAT>(L, C.at(a == 0, a == 1, a == 2), dn);
-      e_m[a] = eps_at<LAT>(L, C.at(-(a == 0), -(a == 1), -(a == 2)), dn);
+      e_p[a] = eps_at<F64>(L, C.at(a == 0, a == 1, a == 2), dn);
+      e_m[a] = eps_at<F64>(L, C.at(-(a == 0), -(a == 1), -(a == 2)), dn);
     } else {
       e_p[a] = e_c;
       e_m[a] = e_c;
@@ -143,18 +186,20 @@ __device__ __forceinline__ void macro_exact(const LatticeDev &L, long long n, co
   m.I = L.qw0 * e_c + L.qw1 * nb;
   m.rho = m.M0 / m.I;
   const double pc = m.rho / 3.0;
+  const double hpc = 0.5 * pc;  // pc (0.5 (e_p - e_m)) = (0.5 pc) (e_p - e_m) exactly
   const double dnf = (double)(n - L.n_force);
   const long long k = C.at(0, 0, 0);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const double grad = 0.5 * (e_p[a] - e_m[a]);
+    m.F[a] = 0.0;
+    if (a >= D) continue;
     double fext = L.g[a];
-    if (L.has_force) fext = fext + force_at<LAT>(L, a, k, dnf);
-    m.F[a] = (a < D) ? fext + pc * grad : 0.0;
+    if (L.has_force) fext = fext + force_at<F64>(L, a, k, dnf);
+    m.F[a] = fext + hpc * (e_p[a] - e_m[a]);
   }
-  if (!L.drag_model) {
+  if (!DRAG || !L.drag_model) {
 #pragma unroll
-    for (int a = 0; a < 3; ++a) m.u[a] = (m.J[a] + 0.5 * m.F[a]) / m.M0;
+    for (int a = 0; a < 3; ++a) m.u[a] = a < D ? __fma_rn(0.5, m.F[a], m.J[a]) / m.M0 : 0.0;
     return;
   }
   // phase-interaction drag F_D = -(b_lin + b_q |u|) u (Ergun-type law of a
@@ -183,43 +228,67 @@ __device__ __forceinline__ void macro_exact(const LatticeDev &L, long long n, co
   }
 }
 
+template <class LAT, bool F64, bool DRAG = true>
+__device__ __forceinline__ void macro_exact(const LatticeDev &L, long long n, const Coords &C, const double *f,
+                                            MacroD &m) {
+  sums_exact<LAT>(f, m);
+  macro_from_sums<LAT, F64, DRAG>(L, n, C, m);
+}
+
+// a . b over the lattice's axes, ascending
 template <class LAT>
-__device__ __forceinline__ double feq_exact(int i, double M0, const double *u, double usq) {
-  double cu = 0.0;
+__device__ __forceinline__ double dot_d(const double *a, const double *b) {
+  double s = a[0] * b[0];
 #pragma unroll
-  for (int a = 0; a < 3; ++a) cu = cu + (double)LAT::c(i, a) * u[a];
-  return LAT::w(i) * M0 * (1.0 + 3.0 * cu + 4.5 * cu * cu - 1.5 * usq);
+  for (int k = 1; k < LAT::D; ++k) s = s + a[k] * b[k];
+  return s;
 }
 
 template <class LAT>
-__device__ __forceinline__ double guo_exact(int i, double cf, const double *u, const double *F,
-                                            double uF) {
-  double cu = 0.0, cF = 0.0;
-#pragma unroll
-  for (int a = 0; a < 3; ++a) cu = cu + (double)LAT::c(i, a) * u[a];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) cF = cF + (double)LAT::c(i, a) * F[a];
-  return cf * LAT::w(i) * (3.0 * (cF - uF) + 9.0 * cu * cF);
+__device__ __forceinline__ double feq_exact(int i, double M0, const double *u, double usq) {
+  const double cu = dot_c<LAT>(i, u);
+  return LAT::w(i) * M0 * (1.0 + 3.0 * cu + 4.5 * cu * cu - 1.5 * usq);
 }
 
 // ---- FP64 step --------------------------------------------------------------
 
-template <class LAT, bool ODD, bool RED>
+// Write f*_i to its slot of the next step.
+template <class LAT, bool ODD>
+__device__ __forceinline__ void put_exact(const LatticeDev &L, const Coords &C, int i, int x, int y, int z,
+                                          double fstar) {
+  const int cx = LAT::c(i, 0), cy = LAT::c(i, 1), cz = LAT::c(i, 2);
+  double *pop = static_cast<double *>(L.pop);
+  if (!ODD || i == 0 || (L.walls && solid_at(L.walls, x, y, z, cx, cy, cz, L.nx, L.ny, L.nz)))
+    pop[(long long)opp_of(i) * L.plane + C.at(0, 0, 0)] = fstar;
+  else
+    pop[(long long)i * L.plane + C.at(cx, cy, cz)] = fstar;
+}
+
+// One thread per cell, cells in linear order over the dense lattice (x
+// fastest): a warp is full whatever nx is, which matters where the FP64 pipe
+// is the bound (rows of 48 cells as 64 lanes cost a third more).
+// EXT: the lattice has the drag law or the closure (a separate instantiation
+// keeps the plain step's registers down).
+template <class LAT, bool ODD, bool RED, bool EXT>
 __global__ void __launch_bounds__(256) step_exact_kernel(const LatticeDev *__restrict__ Lp, int k) {
   constexpr int Q = LAT::Q;
   const LatticeDev &L = *Lp;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  const int z = blockIdx.z;
+  const unsigned nthr = blockDim.x * blockDim.y;
+  const long long idx = (long long)blockIdx.x * nthr + threadIdx.y * blockDim.x + threadIdx.x;
+  const long long plane_cells = (long long)L.nx * L.ny;
   RedAcc acc;
 #pragma unroll
   for (int j = 0; j < kRedWidth; ++j) acc.v[j] = 0.0;
-  const bool inside = x < L.nx && y < L.ny;
+  const bool inside = idx < plane_cells * L.nz;
+  const int z = LAT::D == 3 ? (int)(idx / plane_cells) : 0;
+  const long long rest = LAT::D == 3 ? idx - z * plane_cells : idx;
+  const int y = LAT::D >= 2 ? (int)(rest / L.nx) : 0;
+  const int x = (int)(rest - (long long)y * L.nx);
   const bool fluid = inside && !(L.walls && solid_at(L.walls, x, y, z, 0, 0, 0, L.nx, L.ny, L.nz));
   if (fluid) {
     const long long n = L.n + k;
     const Coords C = make_coords(x, y, z, L.nx, L.ny, L.nz, L.nxp);
-    double *pop = static_cast<double *>(L.pop);
+    const double *pop = static_cast<const double *>(L.pop);
     double f[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
@@ -227,9 +296,9 @@ __global__ void __launch_bounds__(256) step_exact_kernel(const LatticeDev *__res
       f[i] = pop[(long long)a.slot * L.plane + a.cell];
     }
     MacroD m;
-    macro_exact<LAT>(L, n, C, f, m);
-    const double usq = m.u[0] * m.u[0] + m.u[1] * m.u[1] + m.u[2] * m.u[2];
-    const double uF = m.u[0] * m.F[0] + m.u[1] * m.F[1] + m.u[2] * m.F[2];
+    macro_exact<LAT, true, EXT>(L, n, C, f, m);
+    const double usq = dot_d<LAT>(m.u, m.u);
+    const double uF = dot_d<LAT>(m.u, m.F);
     if (RED) {
       acc.v[0] += m.M0;
       acc.v[1] += m.J[0] + 0.5 * m.F[0];
@@ -254,7 +323,7 @@ __global__ void __launch_bounds__(256) step_exact_kernel(const LatticeDev *__res
       acc.v[9] += m.F[2];
     }
     double omega = L.omega, cf = L.cf;
-    if (L.les) {
+    if (EXT && L.les) {
       // Smagorinsky closure: Pi^neq_ab = sum_i xi_ia xi_ib (f_i - f_i^eq),
       // tau_eff = (tau + sqrt(tau^2 + 18 sqrt(2) C^2 |Pi^neq| / M0)) / 2
       double pi[3][3];
@@ -263,48 +332,48 @@ __global__ void __launch_bounds__(256) step_exact_kernel(const LatticeDev *__res
 #pragma unroll
         for (int b = 0; b < 3; ++b) pi[a][b] = 0.0;
 #pragma unroll
-      for (int i = 0; i < Q; ++i) {
+      for (int i = 1; i < Q; ++i) {
         const double fneq = f[i] - feq_exact<LAT>(i, m.M0, m.u, usq);
 #pragma unroll
         for (int a = 0; a < 3; ++a)
 #pragma unroll
-          for (int b = 0; b < 3; ++b) pi[a][b] = pi[a][b] + (double)LAT::c(i, a) * (double)LAT::c(i, b) * fneq;
+          for (int b = a; b < 3; ++b) {
+            const int cc = LAT::c(i, a) * LAT::c(i, b);
+            if (cc != 0) pi[a][b] = cc > 0 ? pi[a][b] + fneq : pi[a][b] - fneq;
+          }
       }
       double q2 = 0.0;
 #pragma unroll
       for (int a = 0; a < 3; ++a)
 #pragma unroll
-        for (int b = 0; b < 3; ++b) q2 = q2 + pi[a][b] * pi[a][b];
+        for (int b = 0; b < 3; ++b) {
+          const double v = a <= b ? pi[a][b] : pi[b][a];
+          q2 = q2 + v * v;
+        }
       const double teff =
           0.5 * (L.tau0 + sqrt(L.tau0 * L.tau0 + 18.0 * sqrt(2.0) * L.les_cs * L.les_cs * sqrt(q2) / m.M0));
       omega = 1.0 / teff;
       cf = 1.0 - 0.5 / teff;
     }
+    const double h = 1.5 * usq;
+    {
+      // rest population: cu = cF = 0
+      const double feq = LAT::w(0) * m.M0 * (1.0 - h);
+      const double S = cf * LAT::w(0) * (3.0 * (0.0 - uF));
+      put_exact<LAT, ODD>(L, C, 0, x, y, z, f[0] + omega * (feq - f[0]) + S);
+    }
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const double feq = feq_exact<LAT>(i, m.M0, m.u, usq);
-      const double S = guo_exact<LAT>(i, cf, m.u, m.F, uF);
-      const double fstar = f[i] + omega * (feq - f[i]) + S;
-      const int cx = LAT::c(i, 0), cy = LAT::c(i, 1), cz = LAT::c(i, 2);
-      long long cell;
-      int slot;
-      if (!ODD || i == 0) {
-        slot = opp_of(i);
-        cell = C.at(0, 0, 0);
-      } else if (L.walls && solid_at(L.walls, x, y, z, cx, cy, cz, L.nx, L.ny, L.nz)) {
-        slot = opp_of(i);
-        cell = C.at(0, 0, 0);
-      } else {
-        slot = i;
-        cell = C.at(cx, cy, cz);
-      }
-      pop[(long long)slot * L.plane + cell] = fstar;
+    for (int i = 1; i < Q; i += 2) {
+      const double wM = LAT::w(i) * m.M0, cw = cf * LAT::w(i);
+      const double cu = dot_c<LAT>(i, m.u), cF = dot_c<LAT>(i, m.F);
+      const double t = 3.0 * cu, q = 4.5 * cu * cu, r = 9.0 * cu * cF;
+      const double ea = wM * (1.0 + t + q - h), eb = wM * (1.0 - t + q - h);
+      const double sa = cw * (3.0 * (cF - uF) + r), sb = cw * (3.0 * (-cF - uF) + r);
+      put_exact<LAT, ODD>(L, C, i, x, y, z, f[i] + omega * (ea - f[i]) + sa);
+      put_exact<LAT, ODD>(L, C, i + 1, x, y, z, f[i + 1] + omega * (eb - f[i + 1]) + sb);
     }
   }
-  if (RED) {
-    const long long b = blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
-    block_reduce_store(acc, L.partials, b);
-  }
+  if (RED) block_reduce_store(acc, L.partials, blockIdx.x);
 }
 
 // ---- moments, initialisation, populations (all storages, FP64 math) ---------
@@ -338,7 +407,8 @@ __global__ void moments_kernel(const LatticeDev *__restrict__ Lp, double *rho, d
 #pragma unroll
   for (int i = 0; i < Q; ++i) f[i] = load_f<LAT>(L, slot_of<LAT>(L, C, odd, i, x, y, z), i);
   MacroD m;
-  macro_exact<LAT>(L, L.n, C, f, m);
+  if (L.storage == 0) macro_exact<LAT, true>(L, L.n, C, f, m);
+  else macro_exact<LAT, false>(L, L.n, C, f, m);
   const double pv = (m.rho - L.rho0) / 3.0;
   if (rho) rho[k] = m.rho;
   if (p) p[k] = pv;
@@ -350,7 +420,7 @@ __global__ void moments_kernel(const LatticeDev *__restrict__ Lp, double *rho, d
   }
 }
 
-template <class LAT>
+template <class LAT, bool F64>
 __global__ void init_kernel(const LatticeDev *__restrict__ Lp, const double *p0, const double *u0,
                             int mode) {
   constexpr int Q = LAT::Q, D = LAT::D;
@@ -378,20 +448,20 @@ __global__ void init_kernel(const LatticeDev *__restrict__ Lp, const double *p0,
     double nb = 0.0;
     for (int a = 0; a < 3; ++a) {
       if (L.quad_axes & (1u << a)) {
-        nb = nb + eps_at<LAT>(L, C.at(a == 0, a == 1, a == 2), dn);
-        nb = nb + eps_at<LAT>(L, C.at(-(a == 0), -(a == 1), -(a == 2)), dn);
+        nb = nb + eps_at<F64>(L, C.at(a == 0, a == 1, a == 2), dn);
+        nb = nb + eps_at<F64>(L, C.at(-(a == 0), -(a == 1), -(a == 2)), dn);
       }
     }
-    mass = rt * (L.qw0 * eps_at<LAT>(L, k, dn) + L.qw1 * nb);
+    mass = rt * (L.qw0 * eps_at<F64>(L, k, dn) + L.qw1 * nb);
   } else {
-    mass = rt * eps_at<LAT>(L, k, dn);
+    mass = rt * eps_at<F64>(L, k, dn);
   }
   double f[Q];
 #pragma unroll
   for (int i = 0; i < Q; ++i) f[i] = feq_exact<LAT>(i, mass, u, usq);
   if (mode & 2) {
     MacroD m;
-    macro_exact<LAT>(L, n, C, f, m);
+    macro_exact<LAT, F64>(L, n, C, f, m);
     for (int a = 0; a < 3; ++a) u[a] = u[a] - 0.5 * m.F[a] / m.M0;
     usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
 #pragma unroll
@@ -423,26 +493,34 @@ __global__ void getpop_kernel(const LatticeDev *__restrict__ Lp, double *out) {
 
 // ---- dispatch ----------------------------------------------------------------
 
-template <class LAT>
-static cudaError_t launch_exact_lat(const LatticeDev *L_dev, bool odd, int red, int k,
-                                    const StepLaunch &ls, cudaStream_t s) {
+template <class LAT, bool EXT>
+static cudaError_t launch_exact_ext(const LatticeDev *L_dev, bool odd, int red, int k, const StepLaunch &ls,
+                                    cudaStream_t s) {
   if (odd) {
-    if (red) step_exact_kernel<LAT, true, true><<<ls.grid, ls.block, 0, s>>>(L_dev, k);
-    else step_exact_kernel<LAT, true, false><<<ls.grid, ls.block, 0, s>>>(L_dev, k);
+    if (red) step_exact_kernel<LAT, true, true, EXT><<<ls.grid, ls.block, 0, s>>>(L_dev, k);
+    else step_exact_kernel<LAT, true, false, EXT><<<ls.grid, ls.block, 0, s>>>(L_dev, k);
   } else {
-    if (red) step_exact_kernel<LAT, false, true><<<ls.grid, ls.block, 0, s>>>(L_dev, k);
-    else step_exact_kernel<LAT, false, false><<<ls.grid, ls.block, 0, s>>>(L_dev, k);
+    if (red) step_exact_kernel<LAT, false, true, EXT><<<ls.grid, ls.block, 0, s>>>(L_dev, k);
+    else step_exact_kernel<LAT, false, false, EXT><<<ls.grid, ls.block, 0, s>>>(L_dev, k);
   }
   return cudaGetLastError();
 }
 
-cudaError_t launch_step_exact(int lattice, const LatticeDev *L_dev, bool odd, int red, int k,
+template <class LAT>
+static cudaError_t launch_exact_lat(const LatticeDev *L_dev, bool ext, bool odd, int red, int k,
+                                    const StepLaunch &ls, cudaStream_t s) {
+  return ext ? launch_exact_ext<LAT, true>(L_dev, odd, red, k, ls, s)
+             : launch_exact_ext<LAT, false>(L_dev, odd, red, k, ls, s);
+}
+
+cudaError_t launch_step_exact(const LatticeDev &h, const LatticeDev *L_dev, bool odd, int red, int k,
                               const StepLaunch &ls, cudaStream_t s) {
-  switch (lattice) {
-    case 0: return launch_exact_lat<D2Q9>(L_dev, odd, red, k, ls, s);
-    case 1: return launch_exact_lat<D3Q19>(L_dev, odd, red, k, ls, s);
-    case 2: return launch_exact_lat<D3Q27>(L_dev, odd, red, k, ls, s);
-    case 3: return launch_exact_lat<D1Q3>(L_dev, odd, red, k, ls, s);
+  const bool ext = h.drag_model || h.les;
+  switch (h.lattice) {
+    case 0: return launch_exact_lat<D2Q9>(L_dev, ext, odd, red, k, ls, s);
+    case 1: return launch_exact_lat<D3Q19>(L_dev, ext, odd, red, k, ls, s);
+    case 2: return launch_exact_lat<D3Q27>(L_dev, ext, odd, red, k, ls, s);
+    case 3: return launch_exact_lat<D1Q3>(L_dev, ext, odd, red, k, ls, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -463,14 +541,21 @@ cudaError_t launch_moments(const LatticeDev &h, const LatticeDev *L_dev, long lo
   return cudaGetLastError();
 }
 
+template <class LAT>
+static void launch_init_lat(const LatticeDev &h, const LatticeDev *L_dev, const double *p0, const double *u0, int mode,
+                            const StepLaunch &ls, cudaStream_t s) {
+  if (h.storage == 0) init_kernel<LAT, true><<<ls.grid, ls.block, 0, s>>>(L_dev, p0, u0, mode);
+  else init_kernel<LAT, false><<<ls.grid, ls.block, 0, s>>>(L_dev, p0, u0, mode);
+}
+
 cudaError_t launch_init(const LatticeDev &h, const LatticeDev *L_dev, long long, const double *p0,
                         const double *u0, int mode, cudaStream_t s) {
   const StepLaunch ls = aux_launch(h);
   switch (h.lattice) {
-    case 0: init_kernel<D2Q9><<<ls.grid, ls.block, 0, s>>>(L_dev, p0, u0, mode); break;
-    case 1: init_kernel<D3Q19><<<ls.grid, ls.block, 0, s>>>(L_dev, p0, u0, mode); break;
-    case 2: init_kernel<D3Q27><<<ls.grid, ls.block, 0, s>>>(L_dev, p0, u0, mode); break;
-    case 3: init_kernel<D1Q3><<<ls.grid, ls.block, 0, s>>>(L_dev, p0, u0, mode); break;
+    case 0: launch_init_lat<D2Q9>(h, L_dev, p0, u0, mode, ls, s); break;
+    case 1: launch_init_lat<D3Q19>(h, L_dev, p0, u0, mode, ls, s); break;
+    case 2: launch_init_lat<D3Q27>(h, L_dev, p0, u0, mode, ls, s); break;
+    case 3: launch_init_lat<D1Q3>(h, L_dev, p0, u0, mode, ls, s); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
