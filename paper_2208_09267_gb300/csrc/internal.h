@@ -118,10 +118,19 @@ cudaError_t launch_moments(const LatticeDev &host_mirror, const LatticeDev *L_de
                            double *rho, double *p, double *u, float *rho_f, float *p_f,
                            float *u_f, cudaStream_t s);
 
+// The same into float outputs for FP32 and FP16 storage, in float-float
+// arithmetic (fields_ff.cu).
+cudaError_t launch_moments_ff(const LatticeDev &host_mirror, const LatticeDev *L_dev, float *rho, float *p, float *u,
+                              cudaStream_t s);
+
 // Equilibrium initialisation at time n (mode bits as lbm_vanse_init_equilibrium);
 // p0 and u0 are device double arrays or null.
 cudaError_t launch_init(const LatticeDev &host_mirror, const LatticeDev *L_dev, long long n_host,
                         const double *p0, const double *u0, int mode, cudaStream_t s);
+
+// The same for FP32 storage, in float-float arithmetic.
+cudaError_t launch_init_ff(const LatticeDev &host_mirror, const LatticeDev *L_dev, const double *p0, const double *u0,
+                           int mode, cudaStream_t s);
 
 // Decoded populations f[cell*Q + i] (double, natural order) into a device buffer.
 cudaError_t launch_get_populations(const LatticeDev &host_mirror, const LatticeDev *L_dev,
