@@ -14,21 +14,29 @@ cudaError_t launch_step_fast_d3q19(const LatticeDev *, int, bool, int, int, cons
 cudaError_t launch_step_fast_d3q27(const LatticeDev *, int, bool, int, int, const StepLaunch &, cudaStream_t);
 cudaError_t launch_step_exact(const LatticeDev &h, const LatticeDev *L_dev, bool odd, int red, int k,
                               const StepLaunch &ls, cudaStream_t s);
-cudaError_t launch_step_row_d2q9(const LatticeDev *, int, bool, int, int, const StepLaunch &, cudaStream_t);
-cudaError_t launch_step_row_d3q19(const LatticeDev *, int, bool, int, int, const StepLaunch &, cudaStream_t);
-cudaError_t launch_step_row_d3q27(const LatticeDev *, int, bool, int, int, const StepLaunch &, cudaStream_t);
-int plan_row_d2q9(int, int, int, int, int, unsigned, StepLaunch &);
-int plan_row_d3q19(int, int, int, int, int, unsigned, StepLaunch &);
-int plan_row_d3q27(int, int, int, int, int, unsigned, StepLaunch &);
+// row-staged kernel, one entry per lattice and storage (step_row_*.cu)
+#define LBM_ROW_DECL(NAME)                                                                              \
+  cudaError_t launch_step_row_##NAME(const LatticeDev *, bool, int, int, const StepLaunch &, cudaStream_t); \
+  int plan_row_##NAME(int, int, int, int, unsigned, StepLaunch &);
+LBM_ROW_DECL(d2q9_f32)
+LBM_ROW_DECL(d2q9_f16)
+LBM_ROW_DECL(d3q19_f32)
+LBM_ROW_DECL(d3q19_f16)
+LBM_ROW_DECL(d3q27_f32)
+LBM_ROW_DECL(d3q27_f16)
+#undef LBM_ROW_DECL
 
 int plan_row_kernel(int lattice, int storage, int nx, int nxp, int ny, int nz, unsigned walls,
                     StepLaunch &ls) {
   ls.row = 0;
   if (storage == 0) return 0;
-  switch (lattice) {
-    case 0: return plan_row_d2q9(storage, nx, nxp, ny, nz, walls, ls);
-    case 1: return plan_row_d3q19(storage, nx, nxp, ny, nz, walls, ls);
-    case 2: return plan_row_d3q27(storage, nx, nxp, ny, nz, walls, ls);
+  switch (lattice * 2 + storage - 1) {
+    case 0: return plan_row_d2q9_f32(nx, nxp, ny, nz, walls, ls);
+    case 1: return plan_row_d2q9_f16(nx, nxp, ny, nz, walls, ls);
+    case 2: return plan_row_d3q19_f32(nx, nxp, ny, nz, walls, ls);
+    case 3: return plan_row_d3q19_f16(nx, nxp, ny, nz, walls, ls);
+    case 4: return plan_row_d3q27_f32(nx, nxp, ny, nz, walls, ls);
+    case 5: return plan_row_d3q27_f16(nx, nxp, ny, nz, walls, ls);
   }
   return 0;
 }
@@ -82,10 +90,13 @@ cudaError_t launch_step(const LatticeDev &h, const LatticeDev *L_dev, long long 
     // since the last step); the row kernel is instantiated for both cases
     // bit 2: phi has no time derivative (a stage layout without d_t phi)
     const int rr = (red ? 1 : 0) | (h.sig_rd != h.sig_wr ? 2 : 0) | (h.has_deps ? 0 : 4);
-    switch (h.lattice) {
-      case 0: return launch_step_row_d2q9(L_dev, h.storage, odd, rr, k, ls, s);
-      case 1: return launch_step_row_d3q19(L_dev, h.storage, odd, rr, k, ls, s);
-      case 2: return launch_step_row_d3q27(L_dev, h.storage, odd, rr, k, ls, s);
+    switch (h.lattice * 2 + h.storage - 1) {
+      case 0: return launch_step_row_d2q9_f32(L_dev, odd, rr, k, ls, s);
+      case 1: return launch_step_row_d2q9_f16(L_dev, odd, rr, k, ls, s);
+      case 2: return launch_step_row_d3q19_f32(L_dev, odd, rr, k, ls, s);
+      case 3: return launch_step_row_d3q19_f16(L_dev, odd, rr, k, ls, s);
+      case 4: return launch_step_row_d3q27_f32(L_dev, odd, rr, k, ls, s);
+      case 5: return launch_step_row_d3q27_f16(L_dev, odd, rr, k, ls, s);
     }
     return cudaErrorInvalidValue;
   }

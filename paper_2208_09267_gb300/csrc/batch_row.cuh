@@ -142,6 +142,8 @@ __global__ void __launch_bounds__(BatchRowCfg<LAT, ST, P>::kThreads, MINB)
     int ny = 1, nz = 1, nxp = 8, y_first = 0, z_first = 0, nyf = 1, R = 1, tpp = 1, rb = 0, re = 0, flags_m = 0;
     unsigned walls = 0;
     const LatticeDev *Lg = nullptr;
+    RowCopies rcp = {};
+    const CtxLane cl(lane);
     int issued_upto = -1;
     RowRuns runs(nitems);
     int j = 0;
@@ -175,6 +177,7 @@ __global__ void __launch_bounds__(BatchRowCfg<LAT, ST, P>::kThreads, MINB)
         R = tile_rows(P, nxp);
         tpp = (nyf + R - 1) / R;
         re = rb + tpp * ((walls & 4u) ? nz - 2 : nz);
+        rcp = row_copies(*Lg, (int)sizeof(ST));
         c0 = make_tile_copy<LAT, ST, ODD, P>(*Lg, lane);
         c1 = make_tile_copy<LAT, ST, ODD, P>(*Lg, lane + 32);
         flags_m = (k >= budget ? 1 : 0) | (REDC && check && k == last ? 4 : 0);
@@ -186,7 +189,7 @@ __global__ void __launch_bounds__(BatchRowCfg<LAT, ST, P>::kThreads, MINB)
       const int lt = r - rb;
       const int tz = lt / tpp, ty = lt - tz * tpp;
       const int y0 = y_first + ty * R, z = z_first + tz, nr = min(R, nyf - ty * R);
-      fill_row_ctx(ctx[s].rc, y0, z, nr, ny, nz, nxp, walls, lane);
+      fill_row_ctx(ctx[s].rc, cl, y0, z, nr, ny, nz, nxp, walls, lane);
       const unsigned bytes =
           __reduce_add_sync(0xffffffffu, tile_copy_bytes(c0, nr, nxp) + tile_copy_bytes(c1, nr, nxp)) +
           (unsigned)kDescBytes;
@@ -202,13 +205,20 @@ __global__ void __launch_bounds__(BatchRowCfg<LAT, ST, P>::kThreads, MINB)
       if (flags_m & 1) {
         if (lane == 0) mbar_arrive(&full[s]);  // nothing to stage: the phase completes
       } else {
-        if (lane == 0) {
-          mbar_arrive_expect_tx(&full[s], bytes);
-          bulk_g2s(&descs[s], Lg, (unsigned)kDescBytes, &full[s]);
+        if (plain_tile(rcp, y0, z, nr)) {
+          if (elect_one()) {
+            issue_plain_tile<LAT, ST, ODD, P>(rcp, smem_u32(stage), smem_u32(&full[s]), bytes, y0, z, nr, true);
+            bulk_g2s(&descs[s], Lg, (unsigned)kDescBytes, &full[s]);
+          }
+        } else {
+          if (lane == 0) {
+            mbar_arrive_expect_tx(&full[s], bytes);
+            bulk_g2s(&descs[s], Lg, (unsigned)kDescBytes, &full[s]);
+          }
+          __syncwarp();
+          issue_tile_copy(c0, stage, &full[s], y0, z, nr, ny, nz, nxp, walls, nxp);
+          issue_tile_copy(c1, stage, &full[s], y0, z, nr, ny, nz, nxp, walls, nxp);
         }
-        __syncwarp();
-        issue_tile_copy(c0, stage, &full[s], y0, z, nr, ny, nz, nxp, walls, nxp);
-        issue_tile_copy(c1, stage, &full[s], y0, z, nr, ny, nz, nxp, walls, nxp);
       }
       issued_upto = j;
       __syncwarp();
@@ -259,8 +269,12 @@ __global__ void __launch_bounds__(BatchRowCfg<LAT, ST, P>::kThreads, MINB)
           const int t = c / ncr, xc = c - t * ncr;
           if constexpr (kPairOK) {
             if (pair) {
-              update_row_pair<LAT, ODD, WALLS, P, false>(Lm, data, t, ctx[s].rc[t], n, dn, dn_force,
-                                                         (xc << 6) + 2 * lane, nullptr);
+              if (Lm.fp16_nearest == 0)
+                update_row_pair<LAT, ODD, WALLS, P, false, true>(Lm, data, t, ctx[s].rc[t], n, dn, dn_force,
+                                                                 (xc << 6) + 2 * lane, nullptr);
+              else
+                update_row_pair<LAT, ODD, WALLS, P, false, false>(Lm, data, t, ctx[s].rc[t], n, dn, dn_force,
+                                                                  (xc << 6) + 2 * lane, nullptr);
               continue;
             }
           }

@@ -28,26 +28,3 @@ cudaError_t launch_step_fast_d3q19(const LatticeDev *L_dev, int storage, bool od
 }
 
 }  // namespace lbm
-
-#include "step_row.cuh"
-
-#ifndef LBM_ROW_MINB_D3Q19
-#define LBM_ROW_MINB_D3Q19 2
-#endif
-
-namespace lbm {
-
-cudaError_t launch_step_row_d3q19(const LatticeDev *L_dev, int storage, bool odd, int red, int k,
-                                  const StepLaunch &ls, cudaStream_t s) {
-  if (storage == 1) return launch_row_t<D3Q19, float, LBM_ROW_MINB_D3Q19>(L_dev, odd, red, k, ls, s);
-  if (storage == 2) return launch_row_t<D3Q19, __half, LBM_ROW_MINB_D3Q19>(L_dev, odd, red, k, ls, s);
-  return cudaErrorInvalidValue;
-}
-
-int plan_row_d3q19(int storage, int nx, int nxp, int ny, int nz, unsigned walls, StepLaunch &ls) {
-  if (storage == 1) return plan_row_t<D3Q19, float, LBM_ROW_MINB_D3Q19>(nx, nxp, ny, nz, walls, ls);
-  if (storage == 2) return plan_row_t<D3Q19, __half, LBM_ROW_MINB_D3Q19>(nx, nxp, ny, nz, walls, ls);
-  return 0;
-}
-
-}  // namespace lbm

@@ -322,23 +322,177 @@ __device__ __forceinline__ void issue_tile_copy(const TileCopy &c, unsigned char
     bulk_g2s(stage + c.dst + run_k * dst_row_bytes, run_src + run_row * row_bytes, run_len * row_bytes, bar);
 }
 
-// The row contexts of the tile (y0, z, nr), written by the producer warp
-// (lanes in parallel) into rc[0 .. nr).
-__device__ __forceinline__ void fill_row_ctx(RowCtx *rc, int y0, int z, int nr, int ny, int nz, int nxp,
-                                             unsigned walls, int lane) {
-  for (int idx = lane; idx < nr * 9; idx += 32) {
-    const int t = idx / 9, e = idx - t * 9;
-    const int dy = e % 3 - 1, dz = e / 3 - 1;
-    rc[t].base[dz + 1][dy + 1] = (wrapi(z + dz, nz) * ny + wrapi(y0 + t + dy, ny)) * nxp;
+// One lane of the calling warp, chosen by the hardware: inside the branch the
+// compiler keeps the copies' operands in uniform registers.
+__device__ __forceinline__ bool elect_one() {
+  unsigned pred;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(pred));
+  return pred != 0;
+}
+
+// What the one-lane copy loops of a lattice need, the same in every lane.
+struct RowCopies {
+  const char *pop, *sig, *eps, *deps;
+  long long plane_bytes;
+  int ny, nz, nxp;
+  unsigned walls;
+};
+
+__device__ __forceinline__ RowCopies row_copies(const LatticeDev &L, int esize) {
+  RowCopies c;
+  c.pop = static_cast<const char *>(L.pop);
+  c.sig = reinterpret_cast<const char *>(L.sig_wr);
+  c.eps = static_cast<const char *>(L.eps);
+  c.deps = L.has_deps ? static_cast<const char *>(L.deps) : nullptr;
+  c.plane_bytes = L.plane * (long long)esize;
+  c.ny = L.ny;
+  c.nz = L.nz;
+  c.nxp = L.nxp;
+  c.walls = L.walls;
+  return c;
+}
+
+// Do the rows y0 - 1 .. y0 + nr lie inside the plane, with no wall layer next
+// to the tile?  Then every block of the tile is one run of rows (planes
+// z - 1 and z + 1 may wrap around) and the one-lane loops below apply.
+__device__ __forceinline__ bool plain_tile(const RowCopies &c, int y0, int z, int nr) {
+  const int m = (c.walls & 2u) ? 2 : 1;
+  if (y0 < m || y0 + nr > c.ny - m) return false;
+  return !(c.walls & 4u) || (z >= 2 && z < c.nz - 2);
+}
+
+// Stage a plain tile: one lane issues the copies of every block in a row,
+// unrolled over compile-time directions.  With the blocks spread over the
+// lanes instead, each copy is issued on its own all the same (its operands
+// are uniform registers), after some 20 instructions that pick the lane.
+template <class LAT, class ST, bool ODD, int PITCH>
+__device__ __forceinline__ void issue_plain_tile(const RowCopies &c, unsigned stage, unsigned bar, unsigned bytes,
+                                                 int y0, int z, int nr, bool merge) {
+  using Lay = RowLayout<LAT, ST, ODD, PITCH>;
+  constexpr int D = LAT::D;
+  auto copy = [&](unsigned dst, const char *src, unsigned n) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "l"(src), "r"(n), "r"(bar)
+                 : "memory");
+  };
+  // n rows of a field from byte offset off, landing at slots of PITCH elements
+  // when the stored pitch differs (one-row tiles: blocks of up to 3 rows)
+  auto rows = [&](unsigned dst, const char *src, int n, unsigned row_bytes, unsigned slot_bytes) {
+    if (merge) {
+      copy(dst, src, (unsigned)n * row_bytes);
+    } else {
+      for (int k = 0; k < n; ++k) copy(dst + k * slot_bytes, src + k * row_bytes, row_bytes);
+    }
+  };
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+  const int dzm = D == 3 ? (z == 0 ? c.nz - 1 : -1) * c.ny : 0, dzp = D == 3 ? (z == c.nz - 1 ? 1 - c.nz : 1) * c.ny : 0;
+  const int r0 = z * c.ny + y0;
+  const unsigned pb = (unsigned)(c.nxp * (int)sizeof(ST));
+  // byte offsets of the neighbour rows; the populations in plane order, so
+  // that every source address is two additions
+  const long long ozm = (long long)dzm * pb, ozp = (long long)dzp * pb;
+  const char *src = c.pop + (long long)r0 * pb;
+#pragma unroll
+  for (int j = 0; j < LAT::Q; ++j) {
+    const int i = ODD ? opp_of(j) : j;  // plane j holds what direction i reads
+    const int cy = ODD ? LAT::c(i, 1) : 0, cz = ODD ? LAT::c(i, 2) : 0;
+    const char *p = src;
+    if (cz > 0) p += ozm;
+    if (cz < 0) p += ozp;
+    if (cy > 0) p -= pb;
+    if (cy < 0) p += pb;
+    copy(stage + i * Lay::kPopBytes, p, (unsigned)nr * pb);
+    src += c.plane_bytes;
   }
-  if (lane < nr) {
-    unsigned solid = 0;
-    if (walls) {
+  const unsigned sb = (unsigned)c.nxp * 2u, fb = (unsigned)c.nxp * 4u;
+  const char *sg = c.sig + (long long)r0 * sb;
+  if (ODD) {
+    rows(stage + Lay::kSigOff + (D == 3 ? 3 * Lay::kSigBytes : 0), sg - sb, nr + 2, sb, Lay::kSigBytes);
+    if (D == 3) {
+      rows(stage + Lay::kSigOff, sg + (long long)dzm * sb - sb, nr + 2, sb, Lay::kSigBytes);
+      rows(stage + Lay::kSigOff + 6 * Lay::kSigBytes, sg + (long long)dzp * sb - sb, nr + 2, sb, Lay::kSigBytes);
+    }
+  } else {
+    copy(stage + Lay::kSigOff, sg, (unsigned)nr * sb);
+  }
+  const long long fo = (long long)r0 * fb, fzm = (long long)dzm * fb, fzp = (long long)dzp * fb;
+#pragma unroll
+  for (int f = 0; f < 2; ++f) {
+    if (f == 1 && !c.deps) break;
+    const char *fld = (f == 0 ? c.eps : c.deps) + fo;
+    const unsigned off = stage + (f == 0 ? Lay::kEpsOff : Lay::kDepsOff);
+    rows(off, fld - fb, nr + 2, fb, Lay::kRowBytes);
+    if (D == 3) {
+      copy(off + 3 * Lay::kRowBytes, fld + fzm, (unsigned)nr * fb);
+      copy(off + 4 * Lay::kRowBytes, fld + fzp, (unsigned)nr * fb);
+    }
+  }
+}
+
+// Write a plain tile's output blocks back (the one-lane counterpart of
+// store_tile_block).
+template <class LAT, class ST, bool ODD, int PITCH>
+__device__ __forceinline__ void store_plain_tile(const RowCopies &c, unsigned ostage, int y0, int z, int nr) {
+  constexpr int D = LAT::D;
+  const int dzm = D == 3 ? (z == 0 ? c.nz - 1 : -1) * c.ny : 0, dzp = D == 3 ? (z == c.nz - 1 ? 1 - c.nz : 1) * c.ny : 0;
+  const unsigned pb = (unsigned)(c.nxp * (int)sizeof(ST));
+  const long long ozm = (long long)dzm * pb, ozp = (long long)dzp * pb;
+  char *dst = const_cast<char *>(c.pop) + (long long)(z * c.ny + y0) * pb;
+#pragma unroll
+  for (int j = 0; j < LAT::Q; ++j) {
+    const int i = ODD ? j : opp_of(j);  // plane j takes what moved along i
+    const int cy = ODD ? LAT::c(i, 1) : 0, cz = ODD ? LAT::c(i, 2) : 0;
+    char *p = dst;
+    if (cz > 0) p += ozp;
+    if (cz < 0) p += ozm;
+    if (cy > 0) p += pb;
+    if (cy < 0) p -= pb;
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(p),
+                 "r"(ostage + i * PITCH * (int)sizeof(ST)), "r"((unsigned)nr * pb)
+                 : "memory");
+    dst += c.plane_bytes;
+  }
+}
+
+// The row contexts of a tile, written by the producer warp (lanes in
+// parallel) into rc[0 .. nr): lane l fills the entries l, l + 32, l + 64 of
+// the tile's 9 nr; which row and neighbour those are is set up once.
+struct CtxLane {
+  int t[3], dy[3], dz[3];
+  __device__ __forceinline__ explicit CtxLane(int lane) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int idx = lane + 32 * k, e = idx % 9;
+      t[k] = idx / 9;
+      dy[k] = e % 3 - 1;
+      dz[k] = e / 3 - 1;
+    }
+  }
+};
+
+__device__ __forceinline__ void fill_row_ctx(RowCtx *rc, const CtxLane &cl, int y0, int z, int nr, int ny, int nz,
+                                             int nxp, unsigned walls, int lane) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    if (k * 32 >= nr * 9) break;
+    if (cl.t[k] < nr)
+      rc[cl.t[k]].base[cl.dz[k] + 1][cl.dy[k] + 1] =
+          (wrapi(z + cl.dz[k], nz) * ny + wrapi(y0 + cl.t[k] + cl.dy[k], ny)) * nxp;
+  }
+  if (walls) {
+    if (lane < nr) {
+      unsigned solid = 0;
 #pragma unroll
       for (int e = 0; e < 9; ++e)
         if (wall_row(walls, y0 + lane + e % 3 - 1, z + e / 3 - 1, ny, nz)) solid |= 1u << e;
+      rc[lane].solid = solid;
     }
-    rc[lane].solid = solid;
+  } else if (lane < nr) {
+    rc[lane].solid = 0;
   }
 }
 
@@ -768,6 +922,21 @@ struct RowCfg {
   static constexpr int kSmemS = kNSS * kInS + kNOut * kOut;
 };
 
+// Position in a ring of n stages: the stage of the current tile and the parity
+// of the pass over the ring it belongs to.
+struct Ring {
+  int s;
+  unsigned pass;
+  __device__ __forceinline__ Ring(int first, int n) : s(first % n), pass((unsigned)(first / n) & 1u) {}
+  __device__ __forceinline__ void step(int by, int n) {
+    s += by;
+    if (s >= n) {
+      s -= n;
+      pass ^= 1u;
+    }
+  }
+};
+
 // Warp-specialised row kernel.  Warps kConsumerWarps .. + kRowProducers - 1
 // are the producers (one by default; producer p takes the block's tiles j =
 // p, p + P, ...): a producer stages tile j into stage j % NSTAGE once the
@@ -822,6 +991,7 @@ __global__ void __launch_bounds__((row_consumers_single<MINB, row_pair_lattice<L
   __shared__ alignas(8) unsigned long long ofull[NOUT > 0 ? NOUT : 1];
   __shared__ alignas(8) unsigned long long oempty[NOUT > 0 ? NOUT : 1];
   __shared__ RowCtx ctx[MAXSTAGE][TILED ? kMaxTileRows : 1];
+  __shared__ int tile_nr[MAXSTAGE];  // rows of the staged tile
   __shared__ volatile int abort_flag;
   extern __shared__ __align__(128) unsigned char stages[];
   const int tid = threadIdx.x;
@@ -886,13 +1056,17 @@ __global__ void __launch_bounds__((row_consumers_single<MINB, row_pair_lattice<L
     const int it0 = (int)blockIdx.x + pw * (int)gridDim.x;
     const int step_y = (int)(stride % (unsigned)tpp), step_z = (int)(stride / (unsigned)tpp);
     int ty = it0 % tpp, tz = it0 / tpp;
+    const RowCopies rcp = row_copies(L, (int)sizeof(ST));
+    const CtxLane cl(lane);
+    const bool merge = spitch == nxp;
     int issued_upto = -1;  // last tile index j whose copies this warp issued
     int j = pw;
-    for (int it = it0; it < ntiles; it += (int)stride, j += kRowProducers) {
-      const int s = j % NSTAGE;
+    Ring ring(pw, NSTAGE);  // tile j's stage and pass, carried along
+    for (int it = it0; it < ntiles; it += (int)stride, j += kRowProducers, ring.step(kRowProducers, NSTAGE)) {
+      const int s = ring.s;
       if (j >= NSTAGE) {
         // the consumers released tile j - NSTAGE from this stage
-        if (!mbar_wait_or_abort(&empty[s], (unsigned)(((j / NSTAGE) - 1) & 1), limit, &abort_flag)) {
+        if (!mbar_wait_or_abort(&empty[s], ring.pass ^ 1u, limit, &abort_flag)) {
           if (lane == 0 && !abort_flag) {
             abort_flag = 1;
             atomicExch(L.status, 1);
@@ -907,15 +1081,21 @@ __global__ void __launch_bounds__((row_consumers_single<MINB, row_pair_lattice<L
         ty -= tpp;
         ++tz;
       }
-      fill_row_ctx(ctx[s], y0, z, nr, ny, nz, nxp, walls, lane);
+      fill_row_ctx(ctx[s], cl, y0, z, nr, ny, nz, nxp, walls, lane);
+      if (lane == 0) tile_nr[s] = nr;
       const unsigned bytes = per_row * (unsigned)nr + fixed;
       __syncwarp();
       if (!withhold) {
-        if (lane == 0) mbar_arrive_expect_tx(&full[s], bytes);
-        __syncwarp();
         unsigned char *stage = stages + s * kInStride;
-        issue_tile_copy(c0, stage, &full[s], y0, z, nr, ny, nz, nxp, walls, spitch);
-        issue_tile_copy(c1, stage, &full[s], y0, z, nr, ny, nz, nxp, walls, spitch);
+        if (plain_tile(rcp, y0, z, nr)) {
+          if (elect_one())
+            issue_plain_tile<LAT, ST, ODD, PITCH>(rcp, smem_u32(stage), smem_u32(&full[s]), bytes, y0, z, nr, merge);
+        } else {
+          if (lane == 0) mbar_arrive_expect_tx(&full[s], bytes);
+          __syncwarp();
+          issue_tile_copy(c0, stage, &full[s], y0, z, nr, ny, nz, nxp, walls, spitch);
+          issue_tile_copy(c1, stage, &full[s], y0, z, nr, ny, nz, nxp, walls, spitch);
+        }
         issued_upto = j;
       }
       __syncwarp();
@@ -930,39 +1110,57 @@ __global__ void __launch_bounds__((row_consumers_single<MINB, row_pair_lattice<L
     // ---------------- storer warp: lane i writes population i's block back
     int cy = 0, cz = 0;
     if (lane < Q) dir_yz<LAT>(lane, cy, cz);
-    int j = 0;
-    for (int it = blockIdx.x; it < ntiles; it += gridDim.x, ++j) {
-      const int o = j % NOUT;
-      if (!mbar_wait_or_abort(&ofull[o], (unsigned)((j / NOUT) & 1), limit, &abort_flag)) {
+    const RowCopies rcp = row_copies(L, (int)sizeof(ST));
+    const int step_y = (int)gridDim.x % tpp, step_z = (int)gridDim.x / tpp;
+    int ty = (int)blockIdx.x % tpp, tz = (int)blockIdx.x / tpp;
+    Ring ring(0, NOUT);
+    for (int it = blockIdx.x; it < ntiles; it += gridDim.x, ring.step(1, NOUT)) {
+      const int o = ring.s;
+      if (!mbar_wait_or_abort(&ofull[o], ring.pass, limit, &abort_flag)) {
         if (lane == 0 && !abort_flag) {
           abort_flag = 1;
           atomicExch(L.status, 1);
         }
         break;
       }
-      const int tz = it / tpp, ty = it - tz * tpp;
       const int y0 = y_first + ty * R, z = z_first + tz, nr = min(R, nyf - ty * R);
-      if (lane < Q) {
-        store_tile_block<LAT, ST, ODD>(L, stages + kInRegion + o * kOutBytes + lane * PITCH * (int)sizeof(ST), lane,
-                                       cy, cz, y0, z, nr, spitch);
+      ty += step_y;
+      tz += step_z;
+      if (ty >= tpp) {
+        ty -= tpp;
+        ++tz;
+      }
+      const unsigned char *ost = stages + kInRegion + o * kOutBytes;
+      if (spitch == L.nxp && plain_tile(rcp, y0, z, nr)) {
+        if (elect_one()) {
+          store_plain_tile<LAT, ST, ODD, PITCH>(rcp, smem_u32(ost), y0, z, nr);
+          bulk_commit();
+          bulk_wait_read_all();
+        }
+      } else if (lane < Q) {
+        store_tile_block<LAT, ST, ODD>(L, ost + lane * PITCH * (int)sizeof(ST), lane, cy, cz, y0, z, nr, spitch);
         bulk_commit();
         bulk_wait_read_all();
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&oempty[o]);
     }
-    if (lane < Q) bulk_wait_all();
+    bulk_wait_all();
   } else {
     // ---------------- consumer warps
     const long long n = L.n + k;
     // steps since the phi and force references, converted once per launch
     const float dn = (float)(n - L.n_eps), dn_force = (float)(n - L.n_force);
     const int ncr = (L.nx + kChunk - 1) / kChunk;  // chunks per row
+    const bool sr = L.fp16_nearest == 0;
+    // small divisions by ncr and the warp count as multiplications (c < 2^8)
+    const unsigned inv_ncr = (65535u + ncr) / (unsigned)ncr, inv_k = (65535u + kConsumerWarps) / (unsigned)kConsumerWarps;
     int rot = 0;  // chunks dealt so far, modulo the consumer warps (all warps agree)
     int j = 0;
-    for (int it = blockIdx.x; it < ntiles; it += gridDim.x, ++j) {
-      const int s = j % NSTAGE;
-      if (!mbar_wait_or_abort(&full[s], (unsigned)((j / NSTAGE) & 1), limit, &abort_flag)) {
+    Ring ring(0, NSTAGE), oring(0, NOUT > 0 ? NOUT : 1);
+    for (int it = blockIdx.x; it < ntiles; it += gridDim.x, ++j, ring.step(1, NSTAGE), oring.step(1, NOUT > 0 ? NOUT : 1)) {
+      const int s = ring.s;
+      if (!mbar_wait_or_abort(&full[s], ring.pass, limit, &abort_flag)) {
         if (lane == 0 && !abort_flag) {
           abort_flag = 1;
           atomicExch(L.status, 1);
@@ -971,9 +1169,9 @@ __global__ void __launch_bounds__((row_consumers_single<MINB, row_pair_lattice<L
       }
       unsigned char *ostage = nullptr;
       if (NOUT > 0) {
-        const int o = j % NOUT;
+        const int o = oring.s;
         // the storer has finished reading tile j - NOUT from this output stage
-        if (j >= NOUT && !mbar_wait_or_abort(&oempty[o], (unsigned)(((j / NOUT) - 1) & 1), limit, &abort_flag)) {
+        if (j >= NOUT && !mbar_wait_or_abort(&oempty[o], oring.pass ^ 1u, limit, &abort_flag)) {
           if (lane == 0 && !abort_flag) {
             abort_flag = 1;
             atomicExch(L.status, 1);
@@ -982,28 +1180,31 @@ __global__ void __launch_bounds__((row_consumers_single<MINB, row_pair_lattice<L
         }
         ostage = stages + kInRegion + o * kOutBytes;
       }
-      const int tz = it / tpp, ty = it - tz * tpp;
-      const int nr = min(R, nyf - ty * R);
       // the tile's chunks (row t, chunk c of the row), dealt round-robin to
       // the consumer warps across tiles so that every warp gets the same share
-      const int nch = nr * ncr;
-      const int first = (warp - rot + kConsumerWarps) % kConsumerWarps;
+      const int nch = tile_nr[s] * ncr;
+      const int first = warp - rot + (warp < rot ? kConsumerWarps : 0);
       const unsigned char *stage = stages + s * kInStride;
       for (int c = first; c < nch; c += kConsumerWarps) {
-        const int t = c / ncr, xc = c - t * ncr;
-        if constexpr (kPair)
-          update_row_pair<LAT, ODD, WALLS, PITCH, (NOUT > 0), TILED>(L, stage, t, ctx[s][t], n, dn, dn_force,
-                                                                     xc * kChunk + 2 * lane, ostage);
-        else
+        const int t = TILED ? (int)((unsigned)c * inv_ncr >> 16) : 0, xc = c - t * ncr;
+        if constexpr (kPair) {
+          if (sr)
+            update_row_pair<LAT, ODD, WALLS, PITCH, (NOUT > 0), true, TILED>(L, stage, t, ctx[s][t], n, dn, dn_force,
+                                                                             xc * kChunk + 2 * lane, ostage);
+          else
+            update_row_pair<LAT, ODD, WALLS, PITCH, (NOUT > 0), false, TILED>(L, stage, t, ctx[s][t], n, dn, dn_force,
+                                                                              xc * kChunk + 2 * lane, ostage);
+        } else
           update_row_chunk<LAT, ST, ODD, RED, WALLS, PITCH, RS, (NOUT > 0), TILED>(
               L, stage, t, ctx[s][t], n, dn, dn_force, xc * kChunk + lane, acc, ostage);
       }
-      rot = (rot + nch) % kConsumerWarps;
+      rot += nch;
+      rot -= (int)((unsigned)rot * inv_k >> 16) * kConsumerWarps;
       if (NOUT > 0) fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) {
         mbar_arrive(&empty[s]);
-        if (NOUT > 0) mbar_arrive(&ofull[j % NOUT]);
+        if (NOUT > 0) mbar_arrive(&ofull[oring.s]);
       }
     }
   }
