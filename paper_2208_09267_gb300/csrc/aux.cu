@@ -8,10 +8,10 @@
 
 namespace lbm {
 
-cudaError_t launch_step_fast_d1q3(const LatticeDev *, int, bool, int, int, const StepLaunch &, cudaStream_t);
-cudaError_t launch_step_fast_d2q9(const LatticeDev *, int, bool, int, int, const StepLaunch &, cudaStream_t);
-cudaError_t launch_step_fast_d3q19(const LatticeDev *, int, bool, int, int, const StepLaunch &, cudaStream_t);
-cudaError_t launch_step_fast_d3q27(const LatticeDev *, int, bool, int, int, const StepLaunch &, cudaStream_t);
+cudaError_t launch_step_fast_d1q3(const LatticeDev *, int, long long, bool, int, int, const StepLaunch &, cudaStream_t);
+cudaError_t launch_step_fast_d2q9(const LatticeDev *, int, long long, bool, int, int, const StepLaunch &, cudaStream_t);
+cudaError_t launch_step_fast_d3q19(const LatticeDev *, int, long long, bool, int, int, const StepLaunch &, cudaStream_t);
+cudaError_t launch_step_fast_d3q27(const LatticeDev *, int, long long, bool, int, int, const StepLaunch &, cudaStream_t);
 cudaError_t launch_step_exact(const LatticeDev &h, const LatticeDev *L_dev, bool odd, int red, int k,
                               const StepLaunch &ls, cudaStream_t s);
 // row-staged kernel, one entry per lattice and storage (step_row_*.cu)
@@ -101,10 +101,10 @@ cudaError_t launch_step(const LatticeDev &h, const LatticeDev *L_dev, long long 
     return cudaErrorInvalidValue;
   }
   switch (h.lattice) {
-    case 0: return launch_step_fast_d2q9(L_dev, h.storage, odd, red, k, ls, s);
-    case 1: return launch_step_fast_d3q19(L_dev, h.storage, odd, red, k, ls, s);
-    case 2: return launch_step_fast_d3q27(L_dev, h.storage, odd, red, k, ls, s);
-    case 3: return launch_step_fast_d1q3(L_dev, h.storage, odd, red, k, ls, s);
+    case 0: return launch_step_fast_d2q9(L_dev, h.storage, h.ncell, odd, red, k, ls, s);
+    case 1: return launch_step_fast_d3q19(L_dev, h.storage, h.ncell, odd, red, k, ls, s);
+    case 2: return launch_step_fast_d3q27(L_dev, h.storage, h.ncell, odd, red, k, ls, s);
+    case 3: return launch_step_fast_d1q3(L_dev, h.storage, h.ncell, odd, red, k, ls, s);
   }
   return cudaErrorInvalidValue;
 }

@@ -98,11 +98,11 @@ __global__ void __launch_bounds__(kBatchBlock) batch_step_kernel(const BatchMemb
       const int y = r % ny;
       const int z = r / ny;
       if (red_here) {
-        if (n & 1) update_cell_fast<LAT, ST, true, true>(L, n, x, y, z, acc, k == 0);
-        else update_cell_fast<LAT, ST, false, true>(L, n, x, y, z, acc, k == 0);
+        if (n & 1) update_cell_fast<LAT, ST, true, true, unsigned>(L, n, x, y, z, acc, k == 0);
+        else update_cell_fast<LAT, ST, false, true, unsigned>(L, n, x, y, z, acc, k == 0);
       } else {
-        if (n & 1) update_cell_fast<LAT, ST, true, false>(L, n, x, y, z, acc, k == 0);
-        else update_cell_fast<LAT, ST, false, false>(L, n, x, y, z, acc, k == 0);
+        if (n & 1) update_cell_fast<LAT, ST, true, false, unsigned>(L, n, x, y, z, acc, k == 0);
+        else update_cell_fast<LAT, ST, false, false, unsigned>(L, n, x, y, z, acc, k == 0);
       }
     }
     if (red_here) {

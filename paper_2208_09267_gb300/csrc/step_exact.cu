@@ -58,6 +58,8 @@ __global__ void __launch_bounds__(256) step_exact_kernel(const LatticeDev *__res
   const int y = LAT::D >= 2 ? (int)(rest / L.nx) : 0;
   const int x = (int)(rest - (long long)y * L.nx);
   const bool fluid = inside && !(L.walls && solid_at(L.walls, x, y, z, 0, 0, 0, L.nx, L.ny, L.nz));
+  chain_wait();
+  chain_release();
   if (fluid) {
     const long long n = L.n + k;
     const Coords C = make_coords(x, y, z, L.nx, L.ny, L.nz, L.nxp);
@@ -195,14 +197,15 @@ __global__ void getpop_kernel(const LatticeDev *__restrict__ Lp, double *out) {
 template <class LAT, bool EXT>
 static cudaError_t launch_exact_ext(const LatticeDev *L_dev, bool odd, int red, int k, const StepLaunch &ls,
                                     cudaStream_t s) {
+  cudaError_t e;
   if (odd) {
-    if (red) step_exact_kernel<LAT, true, true, EXT><<<ls.grid, ls.block, 0, s>>>(L_dev, k);
-    else step_exact_kernel<LAT, true, false, EXT><<<ls.grid, ls.block, 0, s>>>(L_dev, k);
+    if (red) e = launch_chained(step_exact_kernel<LAT, true, true, EXT>, ls.grid, ls.block, 0, s, k > 0, L_dev, k);
+    else e = launch_chained(step_exact_kernel<LAT, true, false, EXT>, ls.grid, ls.block, 0, s, k > 0, L_dev, k);
   } else {
-    if (red) step_exact_kernel<LAT, false, true, EXT><<<ls.grid, ls.block, 0, s>>>(L_dev, k);
-    else step_exact_kernel<LAT, false, false, EXT><<<ls.grid, ls.block, 0, s>>>(L_dev, k);
+    if (red) e = launch_chained(step_exact_kernel<LAT, false, true, EXT>, ls.grid, ls.block, 0, s, k > 0, L_dev, k);
+    else e = launch_chained(step_exact_kernel<LAT, false, false, EXT>, ls.grid, ls.block, 0, s, k > 0, L_dev, k);
   }
-  return cudaGetLastError();
+  return e;
 }
 
 template <class LAT>

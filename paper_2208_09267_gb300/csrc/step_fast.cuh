@@ -174,7 +174,9 @@ struct RedAcc {
 // first: this step is the first since the descriptor's shifts were last
 // committed (a pending refresh applies to it only); the batched kernels,
 // which commit after a replay of several steps, pass false after the first.
-template <class LAT, class ST, bool ODD, bool RED>
+// IDX: index type of a stored cell (unsigned below 2^32 cells: the addresses
+// of an odd step's 2 Q slots and shifts are most of its instructions).
+template <class LAT, class ST, bool ODD, bool RED, class IDX>
 __device__ __forceinline__ void update_cell_fast(const LatticeDev &L, long long n, int x, int y,
                                                  int z, RedAcc &acc, bool first = true) {
   constexpr int Q = LAT::Q;
@@ -183,9 +185,36 @@ __device__ __forceinline__ void update_cell_fast(const LatticeDev &L, long long 
   const unsigned walls = L.walls;
   if (walls && solid_at(walls, x, y, z, 0, 0, 0, nx, ny, nz)) return;
 
-  const Coords C = make_coords(x, y, z, nx, ny, nz, L.nxp);
-  const long long cell = C.at(0, 0, 0);
+  // stored index of the cell at offset (cx, cy, cz), periodic
+  const IDX row = (IDX)L.nxp, slab = (IDX)ny * row;
+  const IDX xo[3] = {(IDX)(x == 0 ? nx - 1 : x - 1), (IDX)x, (IDX)(x == nx - 1 ? 0 : x + 1)};
+  const IDX yo[3] = {(IDX)(y == 0 ? ny - 1 : y - 1) * row, (IDX)y * row, (IDX)(y == ny - 1 ? 0 : y + 1) * row};
+  const IDX zo[3] = {(IDX)(z == 0 ? nz - 1 : z - 1) * slab, (IDX)z * slab, (IDX)(z == nz - 1 ? 0 : z + 1) * slab};
+  auto at = [&](int cx, int cy, int cz) -> IDX { return zo[cz + 1] + yo[cy + 1] + xo[cx + 1]; };
+  const IDX cell = at(0, 0, 0);
   const long long plane = L.plane;
+  // Which neighbours are wall layers: bit (cz+1)*9 + (cy+1)*3 + cx+1.  The
+  // loads and stores below select their address by it instead of branching,
+  // so that they are all in flight together (with a branch per direction a
+  // thread waited for them one after another: an odd step of 150 x 96 x 90
+  // cells with drag and closure took 258 us, an even one 67).
+  unsigned solid = 0;
+  if (ODD && walls) {
+    unsigned xm = 0;
+#pragma unroll
+    for (int o = 0; o < 3; ++o)
+      if ((walls & 1u) && (x + o - 1 <= 0 || x + o - 1 >= nx - 1)) xm |= 1u << o;
+#pragma unroll
+    for (int o = 0; o < 3; ++o) {
+      const bool sz = (walls & 4u) && (z + o - 1 <= 0 || z + o - 1 >= nz - 1);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const bool sy = (walls & 2u) && (y + q - 1 <= 0 || y + q - 1 >= ny - 1);
+        solid |= (sz || sy ? 7u : xm) << (o * 9 + q * 3);
+      }
+    }
+  }
+#define SOLID(cx, cy, cz) ((solid >> (((cz) + 1) * 9 + ((cy) + 1) * 3 + (cx) + 1)) & 1u)
   ST *__restrict__ pop = static_cast<ST *>(L.pop);
   const __half *__restrict__ swr = L.sig_wr;
   const __half *__restrict__ srd = first ? L.sig_rd : swr;
@@ -203,17 +232,20 @@ __device__ __forceinline__ void update_cell_fast(const LatticeDev &L, long long 
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
     const int cx = LAT::c(i, 0), cy = LAT::c(i, 1), cz = LAT::c(i, 2);
-    if (!ODD || i == 0 || (walls && solid_at(walls, x, y, z, -cx, -cy, -cz, nx, ny, nz))) {
+    if (!ODD || i == 0) {
       qraw[i] = PopIO<ST>::ld(pop + (long long)i * plane + cell);
       d[i] = qraw[i] * inv_scale;
       if (kMassFix && reshift) frame = fmaf((float)LAT::w(i), fmaf(-rho0, __half2float(swr[cell]), s_x), frame);
     } else {
-      const long long m = C.at(-cx, -cy, -cz);
-      qraw[i] = PopIO<ST>::ld(pop + (long long)opp_of(i) * plane + m);
+      const bool own = SOLID(-cx, -cy, -cz);
+      const IDX m = own ? cell : at(-cx, -cy, -cz);
+      qraw[i] = PopIO<ST>::ld(pop + (own ? i * plane : opp_of(i) * plane) + m);
       const float sm = __half2float(srd[m]);
-      d[i] = fmaf(qraw[i], inv_scale, fmaf(rho0, sm, -s_x));
+      const float shifted = fmaf(qraw[i], inv_scale, fmaf(rho0, sm, -s_x)), plain = qraw[i] * inv_scale;
+      d[i] = own ? plain : shifted;
       if (kMassFix && reshift)
-        frame = fmaf((float)LAT::w(i), rho0 * (sm - __half2float(swr[m])), frame);
+        frame = fmaf((float)LAT::w(i),
+                     own ? fmaf(-rho0, __half2float(swr[cell]), s_x) : rho0 * (sm - __half2float(swr[m])), frame);
     }
   }
 
@@ -237,18 +269,18 @@ __device__ __forceinline__ void update_cell_fast(const LatticeDev &L, long long 
   const float *__restrict__ deps = static_cast<const float *>(L.deps);
   const bool tv = L.has_deps != 0;
   const float dn = (float)(n - L.n_eps);
-  auto phi = [&](long long m) {
+  auto phi = [&](IDX m) {
     float e = __ldg(eps + m);
     if (tv) e = fmaf(dn, __ldg(deps + m), e);
     return e;
   };
   const float e_c = phi(cell);
-  const float e_xp = phi(C.at(1, 0, 0)), e_xm = phi(C.at(-1, 0, 0));
-  const float e_yp = phi(C.at(0, 1, 0)), e_ym = phi(C.at(0, -1, 0));
+  const float e_xp = phi(at(1, 0, 0)), e_xm = phi(at(-1, 0, 0));
+  const float e_yp = phi(at(0, 1, 0)), e_ym = phi(at(0, -1, 0));
   float e_zp = e_c, e_zm = e_c;
   if (D == 3) {
-    e_zp = phi(C.at(0, 0, 1));
-    e_zm = phi(C.at(0, 0, -1));
+    e_zp = phi(at(0, 0, 1));
+    e_zm = phi(at(0, 0, -1));
   }
 
   // 4. eq. (quad) and eq. (density)
@@ -394,14 +426,16 @@ __device__ __forceinline__ void update_cell_fast(const LatticeDev &L, long long 
     // as the decode does, so that a stored value round-trips
     ST *slot;
     float q;
-    if (!ODD || i == 0 || (walls && solid_at(walls, x, y, z, cx, cy, cz, nx, ny, nz))) {
+    if (!ODD || i == 0) {
       q = ds;
       if (reshift) q += fmaf(-rho0, __half2float(swr[cell]), s_x);
       slot = pop + (long long)opp_of(i) * plane + cell;
     } else {
-      const long long m = C.at(cx, cy, cz);
-      q = ds + fmaf(-rho0, __half2float(swr[m]), s_x);
-      slot = pop + (long long)i * plane + m;
+      const bool own = SOLID(cx, cy, cz);
+      const IDX m = own ? cell : at(cx, cy, cz);
+      const float enc = fmaf(-rho0, __half2float(swr[m]), s_x);
+      q = own && !reshift ? ds : ds + enc;
+      slot = pop + (own ? opp_of(i) * plane : i * plane) + m;
     }
     float v = q;
     if (kMassFix) {
@@ -411,12 +445,14 @@ __device__ __forceinline__ void update_cell_fast(const LatticeDev &L, long long 
     }
     store_pop<ST>(slot, v * scale, rng, sr);
   }
+#undef SOLID
 }
 
 // Sum a thread's accumulators over the block and write them to
-// partials[block * kRedWidth + j] (fixed order, no atomics).
-__device__ __forceinline__ void block_reduce_store(RedAcc &acc, double *partials, long long block) {
-  __shared__ double sm[32][kRedWidth];
+// partials[block * kRedWidth + j] (fixed order, no atomics); sm: one row per
+// warp of shared memory that nothing else uses any more.
+__device__ __forceinline__ void block_reduce_store(RedAcc &acc, double *partials, long long block,
+                                                   double (*sm)[kRedWidth]) {
   const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
   const int nthreads = blockDim.x * blockDim.y * blockDim.z;
   const int lane = tid & 31, warp = tid >> 5;
@@ -436,8 +472,17 @@ __device__ __forceinline__ void block_reduce_store(RedAcc &acc, double *partials
   }
 }
 
-template <class LAT, class ST, bool ODD, bool RED>
-__global__ void __launch_bounds__(256) step_fast_kernel(const LatticeDev *__restrict__ Lp, int k) {
+__device__ __forceinline__ void block_reduce_store(RedAcc &acc, double *partials, long long block) {
+  __shared__ double sm[32][kRedWidth];
+  block_reduce_store(acc, partials, block, sm);
+}
+
+// 128 registers (two blocks of 256 at least): a D3Q19 step of 150 x 96 x 90
+// cells with drag and closure takes 91 us (128 without the limit, 100 at 80
+// registers, 152 with the branching loads); D3Q27 would spill (96 x 64 x 64:
+// 35.5 us, 31.0 without the limit).
+template <class LAT, class ST, bool ODD, bool RED, class IDX>
+__global__ void __launch_bounds__(256, LAT::Q <= 19 ? 2 : 1) step_fast_kernel(const LatticeDev *__restrict__ Lp, int k) {
   const LatticeDev &L = *Lp;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -445,11 +490,38 @@ __global__ void __launch_bounds__(256) step_fast_kernel(const LatticeDev *__rest
   RedAcc acc;
 #pragma unroll
   for (int j = 0; j < kRedWidth; ++j) acc.v[j] = 0.0;
-  if (x < L.nx && y < L.ny) update_cell_fast<LAT, ST, ODD, RED>(L, L.n + k, x, y, z, acc);
+  chain_wait();
+  chain_release();
+  if (x < L.nx && y < L.ny) update_cell_fast<LAT, ST, ODD, RED, IDX>(L, L.n + k, x, y, z, acc);
   if (RED) {
     const long long b = blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
     block_reduce_store(acc, L.partials, b);
   }
+}
+
+template <class LAT, class ST, class IDX>
+cudaError_t launch_step_fast_idx(const LatticeDev *L_dev, bool odd, int red, int k, const StepLaunch &ls,
+                                 cudaStream_t s) {
+  const bool chained = k > 0;
+  if (odd)
+    return red ? launch_chained(step_fast_kernel<LAT, ST, true, true, IDX>, ls.grid, ls.block, 0, s, chained, L_dev, k)
+               : launch_chained(step_fast_kernel<LAT, ST, true, false, IDX>, ls.grid, ls.block, 0, s, chained, L_dev, k);
+  return red ? launch_chained(step_fast_kernel<LAT, ST, false, true, IDX>, ls.grid, ls.block, 0, s, chained, L_dev, k)
+             : launch_chained(step_fast_kernel<LAT, ST, false, false, IDX>, ls.grid, ls.block, 0, s, chained, L_dev, k);
+}
+
+// Host side: one step of a lattice of ncell stored cells.
+template <class LAT>
+cudaError_t launch_step_fast_t(const LatticeDev *L_dev, int storage, long long ncell, bool odd, int red, int k,
+                               const StepLaunch &ls, cudaStream_t s) {
+  const bool wide = ncell > 0xffffffffLL;
+  if (storage == 1)
+    return wide ? launch_step_fast_idx<LAT, float, long long>(L_dev, odd, red, k, ls, s)
+                : launch_step_fast_idx<LAT, float, unsigned>(L_dev, odd, red, k, ls, s);
+  if (storage == 2)
+    return wide ? launch_step_fast_idx<LAT, __half, long long>(L_dev, odd, red, k, ls, s)
+                : launch_step_fast_idx<LAT, __half, unsigned>(L_dev, odd, red, k, ls, s);
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace lbm
