@@ -216,8 +216,8 @@ __global__ void __launch_bounds__(BatchRowCfg<LAT, ST, P>::kThreads, MINB)
             bulk_g2s(&descs[s], Lg, (unsigned)kDescBytes, &full[s]);
           }
           __syncwarp();
-          issue_tile_copy(c0, stage, &full[s], y0, z, nr, ny, nz, nxp, walls, nxp);
-          issue_tile_copy(c1, stage, &full[s], y0, z, nr, ny, nz, nxp, walls, nxp);
+          issue_tile_copy<false>(c0, stage, &full[s], y0, z, nr, ny, nz, nxp, walls, nxp);
+          issue_tile_copy<false>(c1, stage, &full[s], y0, z, nr, ny, nz, nxp, walls, nxp);
         }
       }
       issued_upto = j;
@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(BatchRowCfg<LAT, ST, P>::kThreads, MINB)
       }
       const int flags = ctx[s].flags;
       if (!(flags & 1)) {
-        const unsigned char *data = stages + s * kStage;
+        unsigned char *data = stages + s * kStage;
         const LatticeDev &Lm = descs[s];
         const int m = ctx[s].member;
         const bool red = REDC && (flags & 4) != 0;
@@ -271,10 +271,10 @@ __global__ void __launch_bounds__(BatchRowCfg<LAT, ST, P>::kThreads, MINB)
             if (pair) {
               if (Lm.fp16_nearest == 0)
                 update_row_pair<LAT, ODD, WALLS, P, false, true>(Lm, data, t, ctx[s].rc[t], n, dn, dn_force,
-                                                                 (xc << 6) + 2 * lane, nullptr);
+                                                                 (xc << 6) + 2 * lane);
               else
                 update_row_pair<LAT, ODD, WALLS, P, false, false>(Lm, data, t, ctx[s].rc[t], n, dn, dn_force,
-                                                                  (xc << 6) + 2 * lane, nullptr);
+                                                                  (xc << 6) + 2 * lane);
               continue;
             }
           }

@@ -42,33 +42,22 @@ namespace lbm {
 #ifndef LBM_ROW_CONSUMERS
 #define LBM_ROW_CONSUMERS 7
 #endif
-#ifndef LBM_ROW_CONSUMERS_F16
-#define LBM_ROW_CONSUMERS_F16 6
-#endif
 #ifndef LBM_ROW_PRODUCERS
 #define LBM_ROW_PRODUCERS 1  // producer warps per block of the single-lattice row kernel (1 or 2)
-#endif
-#ifndef LBM_ROW_OUTS_F16
-#define LBM_ROW_OUTS_F16 1  // FP16 rows written back through output stages (0: direct stores)
 #endif
 // Consumer warps per block (+ one producer warp).  Two blocks per SM (MINB
 // 2) take 7: every SM sub-partition then holds four warps of up to 128
 // registers.  Where a stage is too large for two blocks per SM (MINB 1: rows
-// of 512 cells, D3Q27) one block takes 15, so the SM keeps 16 warps.  FP16
-// D2Q9/D3Q19 blocks also have a storer warp and update two cells per lane
-// (more live registers): 6 consumers (14 with MINB 1) keep them at 16 warps
-// per SM, 128 registers each.
-template <int MINB, bool PAIR = false>
-constexpr int row_consumers() {
-  return PAIR ? (MINB == 1 ? 14 : LBM_ROW_CONSUMERS_F16) : (MINB == 1 ? 15 : LBM_ROW_CONSUMERS);
-}
+// of 512 cells, D3Q27) one block takes 15, so the SM keeps 16 warps.
 template <int MINB>
-constexpr int row_threads() { return (row_consumers<MINB>() + 1) * 32; }
+constexpr int row_consumers() {
+  return MINB == 1 ? 15 : LBM_ROW_CONSUMERS;
+}
 // the single-lattice kernel: producer warps per block, and consumers (one
 // fewer per extra producer, so that the block keeps its warp count)
 constexpr int kRowProducers = LBM_ROW_PRODUCERS;
-template <int MINB, bool PAIR>
-constexpr int row_consumers_single() { return row_consumers<MINB, PAIR>() - (kRowProducers - 1); }
+template <int MINB>
+constexpr int row_consumers_single() { return row_consumers<MINB>() - (kRowProducers - 1); }
 // FP16 plain steps of D2Q9/D3Q19 update two adjacent cells per lane
 // (update_row_pair); D3Q27's larger state would spill
 template <class LAT, class ST>
@@ -105,6 +94,27 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned by
           smem_u32(dst)),
       "l"(src), "r"(bytes), "r"(smem_u32(bar))
       : "memory");
+}
+
+// Bulk copy of `bytes` from shared to global memory (both 16-byte aligned, a
+// multiple of 16 bytes), tracked in this thread's bulk async-group.
+__device__ __forceinline__ void bulk_s2g(void *dst, const void *src, unsigned bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)),
+               "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+// wait until all but the N latest of this thread's bulk-store groups have
+// read their shared-memory source
+template <int N>
+__device__ __forceinline__ void bulk_wait_read() {
+  asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
+}
+// wait until this thread's bulk stores have completed
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+// make this thread's shared-memory writes visible to the bulk-copy engine
+__device__ __forceinline__ void fence_proxy_async_smem() {
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
 __device__ __forceinline__ bool mbar_try_wait(unsigned long long *bar, unsigned parity) {
@@ -271,7 +281,15 @@ __device__ __forceinline__ unsigned tile_copy_bytes(const TileCopy &c, int nr, i
 // Source rows inside the lattice, in one plane, with no wall substitution
 // (every block but those at a periodic edge or next to a wall) go as one
 // copy (or one per row when the two row sizes differ); the others are
-// split into runs of rows consecutive in both places.
+// split into runs of rows consecutive in both places.  STORE: the same runs
+// back from the stage to where they came from (bulk stores, no barrier).
+template <bool STORE>
+__device__ __forceinline__ void move_rows(unsigned char *stage, const char *mem, unsigned bytes,
+                                          unsigned long long *bar) {
+  if (STORE) bulk_s2g(const_cast<char *>(mem), stage, bytes);
+  else bulk_g2s(stage, mem, bytes, bar);
+}
+template <bool STORE>
 __device__ __forceinline__ void issue_tile_copy(const TileCopy &c, unsigned char *stage, unsigned long long *bar,
                                                 int y0, int z, int nr, int ny, int nz, int nxp, unsigned walls,
                                                 int dst_pitch) {
@@ -288,9 +306,9 @@ __device__ __forceinline__ void issue_tile_copy(const TileCopy &c, unsigned char
     const char *src = c.src + ((long long)zs * ny + ys) * row_bytes;
     unsigned char *dst = stage + c.dst;
     if (merge) {
-      bulk_g2s(dst, src, (unsigned)n * row_bytes, bar);
+      move_rows<STORE>(dst, src, (unsigned)n * row_bytes, bar);
     } else {
-      for (int k = 0; k < n; ++k) bulk_g2s(dst + k * dst_row_bytes, src + k * row_bytes, row_bytes, bar);
+      for (int k = 0; k < n; ++k) move_rows<STORE>(dst + k * dst_row_bytes, src + k * row_bytes, row_bytes, bar);
     }
     return;
   }
@@ -312,14 +330,14 @@ __device__ __forceinline__ void issue_tile_copy(const TileCopy &c, unsigned char
       continue;
     }
     if (run_len)
-      bulk_g2s(stage + c.dst + run_k * dst_row_bytes, run_src + run_row * row_bytes, run_len * row_bytes, bar);
+      move_rows<STORE>(stage + c.dst + run_k * dst_row_bytes, run_src + run_row * row_bytes, run_len * row_bytes, bar);
     run_src = src;
     run_row = row;
     run_k = k;
     run_len = 1;
   }
   if (run_len)
-    bulk_g2s(stage + c.dst + run_k * dst_row_bytes, run_src + run_row * row_bytes, run_len * row_bytes, bar);
+    move_rows<STORE>(stage + c.dst + run_k * dst_row_bytes, run_src + run_row * row_bytes, run_len * row_bytes, bar);
 }
 
 // One lane of the calling warp, chosen by the hardware: inside the branch the
@@ -433,10 +451,11 @@ __device__ __forceinline__ void issue_plain_tile(const RowCopies &c, unsigned st
   }
 }
 
-// Write a plain tile's output blocks back (the one-lane counterpart of
-// store_tile_block).
+// Store a plain tile's population blocks back to where issue_plain_tile
+// loaded them from.
 template <class LAT, class ST, bool ODD, int PITCH>
-__device__ __forceinline__ void store_plain_tile(const RowCopies &c, unsigned ostage, int y0, int z, int nr) {
+__device__ __forceinline__ void store_plain_tile(const RowCopies &c, unsigned stage, int y0, int z, int nr) {
+  using Lay = RowLayout<LAT, ST, ODD, PITCH>;
   constexpr int D = LAT::D;
   const int dzm = D == 3 ? (z == 0 ? c.nz - 1 : -1) * c.ny : 0, dzp = D == 3 ? (z == c.nz - 1 ? 1 - c.nz : 1) * c.ny : 0;
   const unsigned pb = (unsigned)(c.nxp * (int)sizeof(ST));
@@ -444,15 +463,15 @@ __device__ __forceinline__ void store_plain_tile(const RowCopies &c, unsigned os
   char *dst = const_cast<char *>(c.pop) + (long long)(z * c.ny + y0) * pb;
 #pragma unroll
   for (int j = 0; j < LAT::Q; ++j) {
-    const int i = ODD ? j : opp_of(j);  // plane j takes what moved along i
+    const int i = ODD ? opp_of(j) : j;
     const int cy = ODD ? LAT::c(i, 1) : 0, cz = ODD ? LAT::c(i, 2) : 0;
     char *p = dst;
-    if (cz > 0) p += ozp;
-    if (cz < 0) p += ozm;
-    if (cy > 0) p += pb;
-    if (cy < 0) p -= pb;
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(p),
-                 "r"(ostage + i * PITCH * (int)sizeof(ST)), "r"((unsigned)nr * pb)
+    if (cz > 0) p += ozm;
+    if (cz < 0) p += ozp;
+    if (cy > 0) p -= pb;
+    if (cy < 0) p += pb;
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(p), "r"(stage + i * Lay::kPopBytes),
+                 "r"((unsigned)nr * pb)
                  : "memory");
     dst += c.plane_bytes;
   }
@@ -474,10 +493,14 @@ struct CtxLane {
   }
 };
 
+// NB: with the neighbour rows (else the own row only, all that an in-place
+// update without a pending shift change asks for).
+template <bool NB = true>
 __device__ __forceinline__ void fill_row_ctx(RowCtx *rc, const CtxLane &cl, int y0, int z, int nr, int ny, int nz,
                                              int nxp, unsigned walls, int lane) {
+  if (!NB && lane < nr) rc[lane].base[1][1] = (z * ny + y0 + lane) * nxp;
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
+  for (int k = 0; NB && k < 3; ++k) {
     if (k * 32 >= nr * 9) break;
     if (cl.t[k] < nr)
       rc[cl.t[k]].base[cl.dz[k] + 1][cl.dy[k] + 1] =
@@ -501,15 +524,15 @@ __device__ __forceinline__ void fill_row_ctx(RowCtx *rc, const CtxLane &cl, int 
 // RS: the step after a phi refresh decodes with the old shift and encodes
 // with the new one ("reshift").  0: no refresh pending, 1: pending (both
 // known at launch), 2: read it from the descriptor.
-// OUTS: the updated populations go to the output stage `ostage` in shared
-// memory (row i holds f*_i at the position of its storage cell in the
-// destination row) instead of straight to global memory; a storer warp
-// writes the rows back with bulk copies.
-template <class LAT, class ST, bool ODD, bool RED, bool WALLS, int PITCH, int RS = 2, bool OUTS = false,
+// INPLACE: the updated populations overwrite the staged ones (f*_i goes where
+// f_opp(i) was read: the AA pattern writes the slots it reads) instead of
+// going straight to global memory; a storer warp writes the rows back with
+// bulk copies.
+template <class LAT, class ST, bool ODD, bool RED, bool WALLS, int PITCH, int RS = 2, bool INPLACE = false,
           bool TILED = true>
-__device__ __forceinline__ void update_row_chunk(const LatticeDev &L, const unsigned char *stage, int t,
+__device__ __forceinline__ void update_row_chunk(const LatticeDev &L, unsigned char *stage, int t,
                                                  const RowCtx &rc, long long n, float dn, float dn_force,
-                                                 int x, RedAcc &acc, unsigned char *ostage = nullptr) {
+                                                 int x, RedAcc &acc) {
   using Lay = RowLayout<LAT, ST, ODD, PITCH>;
   constexpr int Q = LAT::Q, D = LAT::D;
   // FP16 stores deviations times 2^k.  The update below runs in those
@@ -711,7 +734,7 @@ __device__ __forceinline__ void update_row_chunk(const LatticeDev &L, const unsi
   const float enc_own = reshift ? fmaf(-rho0, sig_own, s_x) : 0.f;
   SRng rng((unsigned)cell, n);
   const bool sr = L.fp16_nearest == 0;
-  ST *orow = OUTS ? reinterpret_cast<ST *>(ostage) + tt * sp : nullptr;
+  ST *orow = INPLACE ? reinterpret_cast<ST *>(stage) + tt * sp : nullptr;
   // encode population i (compile-time index) with post-collision deviation
   // DSTAR (storage units): P_ = its slot, V_ = the value to store against
   // the shift of the cell whose memory holds it
@@ -723,7 +746,7 @@ __device__ __forceinline__ void update_row_chunk(const LatticeDev &L, const unsi
     const float ds_ = (DSTAR);                                                                     \
     if (OWN_DST(i)) {                                                                              \
       V_ = reshift ? fmaf(enc_own, sc, ds_) : ds_;                                                 \
-      P_ = OUTS ? orow + (i) * PITCH + x : (pop + opp_of(i) * plane) + cell;                   \
+      P_ = INPLACE ? orow + opp_of(i) * PITCH + x : (pop + opp_of(i) * plane) + cell;              \
     } else {                                                                                       \
       const int xm_ = xs[1 + cx_];                                                                 \
       float enc_;                                                                                  \
@@ -732,7 +755,7 @@ __device__ __forceinline__ void update_row_chunk(const LatticeDev &L, const unsi
       else                                                                                         \
         enc_ = fmaf(-rho0, SIG_AT(cy_, cz_, xm_), s_x);                                            \
       V_ = fmaf(enc_, sc, ds_);                                                                    \
-      P_ = OUTS ? orow + (i) * PITCH + xm_                                                        \
+      P_ = INPLACE ? orow + opp_of(i) * PITCH + xm_                                               \
                 : (pop + (i) * plane) + (rc.base[1 + cz_][1 + cy_] + xm_);                         \
     }                                                                                              \
   }
@@ -834,92 +857,30 @@ __device__ __forceinline__ bool mbar_wait_or_abort(unsigned long long *bar, unsi
   return false;
 }
 
-// Bulk copy of `bytes` from shared to global memory (both 16-byte aligned, a
-// multiple of 16 bytes), tracked in this thread's bulk async-group.
-__device__ __forceinline__ void bulk_s2g(void *dst, const void *src, unsigned bytes) {
-  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)),
-               "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-// wait until this thread's bulk stores have read their shared-memory source
-__device__ __forceinline__ void bulk_wait_read_all() {
-  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-}
-// wait until this thread's bulk stores have completed
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-// make this thread's shared-memory writes visible to the bulk-copy engine
-__device__ __forceinline__ void fence_proxy_async_smem() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
-// Write population i's output block of the tile (y0, z, nr) back (storer
-// lane i; block row t at t * src_pitch elements): row t goes to row (y0 + t
-// + c_iy, z + c_iz) of plane i at odd steps (i > 0) unless that row is a
-// wall layer, else to the own row of plane opp(i); one bulk store per run of
-// rows consecutive in both places.
-template <class LAT, class ST, bool ODD>
-__device__ __forceinline__ void store_tile_block(const LatticeDev &L, const unsigned char *oblock, int i, int cy,
-                                                 int cz, int y0, int z, int nr, int src_pitch) {
-  const int ny = L.ny, nz = L.nz, nxp = L.nxp;
-  const unsigned walls = L.walls;
-  const long long plane_bytes = L.plane * (long long)sizeof(ST);
-  char *pop = static_cast<char *>(L.pop);
-  const unsigned row_bytes = (unsigned)nxp * (unsigned)sizeof(ST);
-  const unsigned src_row_bytes = (unsigned)src_pitch * (unsigned)sizeof(ST);
-  const bool merge = src_row_bytes == row_bytes;
-  const bool moves = ODD && i != 0;
-  char *run_dst = nullptr;
-  int run_t = 0, run_len = 0;
-  long long run_row = 0;
-  for (int t = 0; t < nr; ++t) {
-    const int y = y0 + t;
-    const bool to_nb = moves && !(walls && wall_row(walls, y + cy, z + cz, ny, nz));
-    const int yy = to_nb ? wrapi(y + cy, ny) : y, zz = to_nb ? wrapi(z + cz, nz) : z;
-    char *dst = pop + (to_nb ? i : opp_of(i)) * plane_bytes;
-    const long long row = (long long)zz * ny + yy;
-    if (run_len && merge && dst == run_dst && row == run_row + run_len) {
-      ++run_len;
-      continue;
-    }
-    if (run_len) bulk_s2g(run_dst + run_row * row_bytes, oblock + run_t * src_row_bytes, run_len * row_bytes);
-    run_dst = dst;
-    run_row = row;
-    run_t = t;
-    run_len = 1;
-  }
-  if (run_len) bulk_s2g(run_dst + run_row * row_bytes, oblock + run_t * src_row_bytes, run_len * row_bytes);
-}
-
-// Shape of one row kernel instantiation.  FP16 rows are written back
-// through two output stages in shared memory by bulk copies (fewer
-// instructions per cell than scattered 2-byte stores: measured -8 % on the
-// odd step, +2 % GLUPS at 256^3), where that fits with at least two input
-// stages; FP32 keeps three input stages and stores directly (with output
-// staging it would drop to two input stages: measured 0.78 instead of 0.88
-// of the copy bandwidth).
+// Shape of one row kernel instantiation (FP32: the consumers store straight
+// to global memory).
 template <class LAT, class ST, int P, int MINB>
 struct RowCfg {
   static constexpr int kIn = RowLayout<LAT, ST, true, P>::kStageBytes;  // the odd step's (larger) stage
-  static constexpr int kOut = (LAT::Q * P * (int)sizeof(ST) + 127) / 128 * 128;
   static constexpr int kBudget = MINB > 1 ? 110 * 1024 : 216 * 1024;
   static constexpr int kMaxIn = MINB > 1 ? 3 : 6;
-  static constexpr int kInWithOut = (kBudget - 2 * kOut) / kIn;
-  static constexpr bool kOuts = LBM_ROW_OUTS_F16 && sizeof(ST) == 2 && kInWithOut >= 2;
-  static constexpr int kInOnly = kBudget / kIn;
-  static constexpr int kNS = kOuts ? (kInWithOut < kMaxIn ? kInWithOut : kMaxIn) : (kInOnly < kMaxIn ? kInOnly : kMaxIn);
-  static constexpr int kNOut = kOuts ? 2 : 0;
-  static constexpr int kConsumers = row_consumers_single<MINB, row_pair_lattice<LAT, ST>()>();
-  static constexpr int kThreads = (kConsumers + kRowProducers + (kOuts ? 1 : 0)) * 32;
-  static constexpr int kSmem = kNS * kIn + kNOut * kOut;
+  static constexpr int kNS = kBudget / kIn < kMaxIn ? kBudget / kIn : kMaxIn;
+  static constexpr int kConsumers = row_consumers_single<MINB>();
+  static constexpr int kThreads = (kConsumers + kRowProducers) * 32;
+  static constexpr int kSmem = kNS * kIn;
   // static phi (no d_t phi blocks): a stage ends where the d_t phi blocks
   // would start; one-block-per-SM shapes then fit more stages in up to
   // 226 KB (D3Q27 at pitch 512: 3 instead of 2)
   static constexpr int kInS = RowLayout<LAT, ST, true, P>::kDepsOff;
   static constexpr int kBudgetS = MINB > 1 ? kBudget : 226 * 1024;
-  static constexpr int kNSS0 = (kBudgetS - kNOut * kOut) / kInS;
+  static constexpr int kNSS0 = kBudgetS / kInS;
   static constexpr int kNSS = kNSS0 > kNS ? (kNSS0 < kMaxIn ? kNSS0 : kMaxIn) : kNS;
-  static constexpr int kSmemS = kNSS * kInS + kNOut * kOut;
+  static constexpr int kSmemS = kNSS * kInS;
+};
+
+template <bool V>
+struct Bool {
+  static constexpr bool value = V;
 };
 
 // Position in a ring of n stages: the stage of the current tile and the parity
@@ -948,34 +909,22 @@ struct Ring {
 // besides the copies.  The consumer warps wait on the full barrier, update
 // their chunks of the tile's rows and release the stage, one arrival per
 // warp.
-// NOUT > 0: the consumers write the updated tile into output stage j % NOUT
-// (after the storer has released it: oempty), then arrive on ofull; the
-// storer warp (the one after the producers) waits on ofull, copies the Q output blocks
-// to their destination rows with bulk copies (lane i: population i), waits
-// until the copies have read the stage and releases it.  No block-wide
-// barrier is taken inside the loop.
+// No block-wide barrier is taken inside the loop.
 // TUNED = false: row_consumers_single() consumer warps and RowCfg's input
 // stages (kNS; kNSS when the launch asks for the static-phi layout),
 // compile-time constants (the default shape).  TUNED = true: the launch
-// chooses the consumer warps (blockDim.x / 32 minus the producer and storer
-// warps, at most the default) and the input stages `nstage` (2 <= nstage <=
+// chooses the consumer warps (blockDim.x / 32 minus the producer, at most
+// the default) and the input stages `nstage` (2 <= nstage <=
 // MAXSTAGE), the autotuner's knobs; this generic form costs 2-5 % at the
 // default shape (measured), so it runs only when a tuned shape differs from
 // the default, and only for plain steps.
-template <class LAT, class ST, bool ODD, bool RED, bool WALLS, int PITCH, int MAXSTAGE, int MINB, int RS, int NOUT,
+template <class LAT, class ST, bool ODD, bool RED, bool WALLS, int PITCH, int MAXSTAGE, int MINB, int RS,
           bool TILED, bool TUNED = false>
-__global__ void __launch_bounds__((row_consumers_single<MINB, row_pair_lattice<LAT, ST>()>() + kRowProducers +
-                                   (NOUT ? 1 : 0)) * 32, MINB)
+__global__ void __launch_bounds__((row_consumers_single<MINB>() + kRowProducers) * 32, MINB)
     step_row_kernel(const LatticeDev *__restrict__ Lp, int k, int nstage, int lay_static) {
-  constexpr int Q = LAT::Q;
   using Lay = RowLayout<LAT, ST, ODD, PITCH>;
-  constexpr int kOutBytes = (Q * PITCH * (int)sizeof(ST) + 127) / 128 * 128;
-  // FP16 plain steps of D2Q9/D3Q19 update two adjacent cells per lane
-  // (update_row_pair: bit-identical results, fewer instructions per cell)
-  constexpr bool kPair = row_pair_lattice<LAT, ST>() && !RED && RS == 0;
-  constexpr int kChunk = kPair ? 64 : 32;
-  const int kConsumerWarps = TUNED ? (int)(blockDim.x >> 5) - kRowProducers - (NOUT ? 1 : 0)
-                                   : row_consumers_single<MINB, row_pair_lattice<LAT, ST>()>();
+  constexpr int kChunk = 32;
+  const int kConsumerWarps = TUNED ? (int)(blockDim.x >> 5) - kRowProducers : row_consumers_single<MINB>();
   // input stages: MAXSTAGE is the static-phi count (RowCfg::kNSS); with
   // lay_static (phi without d_t phi, set by the launch) stages end where the
   // d_t phi blocks would start
@@ -983,13 +932,9 @@ __global__ void __launch_bounds__((row_consumers_single<MINB, row_pair_lattice<L
   const bool stat = Cfg::kNSS > Cfg::kNS && lay_static != 0;
   const int NSTAGE = TUNED ? nstage : (stat ? Cfg::kNSS : Cfg::kNS);
   const int kInStride = stat ? Lay::kDepsOff : Lay::kStageBytes;
-  const int kInRegion = NSTAGE * (stat ? RowLayout<LAT, ST, true, PITCH>::kDepsOff
-                                       : RowLayout<LAT, ST, true, PITCH>::kStageBytes);
   __shared__ LatticeDev Ls;
   __shared__ alignas(8) unsigned long long full[MAXSTAGE];
   __shared__ alignas(8) unsigned long long empty[MAXSTAGE];
-  __shared__ alignas(8) unsigned long long ofull[NOUT > 0 ? NOUT : 1];
-  __shared__ alignas(8) unsigned long long oempty[NOUT > 0 ? NOUT : 1];
   __shared__ RowCtx ctx[MAXSTAGE][TILED ? kMaxTileRows : 1];
   __shared__ int tile_nr[MAXSTAGE];  // rows of the staged tile
   __shared__ volatile int abort_flag;
@@ -1005,10 +950,6 @@ __global__ void __launch_bounds__((row_consumers_single<MINB, row_pair_lattice<L
     for (int s = 0; s < NSTAGE; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], kConsumerWarps);
-    }
-    for (int o = 0; o < NOUT; ++o) {
-      mbar_init(&ofull[o], kConsumerWarps);
-      mbar_init(&oempty[o], 1);
     }
     abort_flag = 0;
     mbar_fence_init();
@@ -1036,6 +977,8 @@ __global__ void __launch_bounds__((row_consumers_single<MINB, row_pair_lattice<L
   RedAcc acc;
 #pragma unroll
   for (int j = 0; j < kRedWidth; ++j) acc.v[j] = 0.0;
+  chain_wait();
+  chain_release();
 
   if (warp >= kConsumerWarps && warp < kConsumerWarps + kRowProducers) {
     // ---------------- producer warp p: tiles j = p, p + P, p + 2P, ... of the
@@ -1093,8 +1036,8 @@ __global__ void __launch_bounds__((row_consumers_single<MINB, row_pair_lattice<L
         } else {
           if (lane == 0) mbar_arrive_expect_tx(&full[s], bytes);
           __syncwarp();
-          issue_tile_copy(c0, stage, &full[s], y0, z, nr, ny, nz, nxp, walls, spitch);
-          issue_tile_copy(c1, stage, &full[s], y0, z, nr, ny, nz, nxp, walls, spitch);
+          issue_tile_copy<false>(c0, stage, &full[s], y0, z, nr, ny, nz, nxp, walls, spitch);
+          issue_tile_copy<false>(c1, stage, &full[s], y0, z, nr, ny, nz, nxp, walls, spitch);
         }
         issued_upto = j;
       }
@@ -1106,59 +1049,17 @@ __global__ void __launch_bounds__((row_consumers_single<MINB, row_pair_lattice<L
       for (int jj = issued_upto; jj >= 0 && jj > issued_upto - NSTAGE * kRowProducers; jj -= kRowProducers)
         mbar_wait_bounded(&full[jj % NSTAGE], (unsigned)((jj / NSTAGE) & 1));
     }
-  } else if (NOUT > 0 && warp == kConsumerWarps + kRowProducers) {
-    // ---------------- storer warp: lane i writes population i's block back
-    int cy = 0, cz = 0;
-    if (lane < Q) dir_yz<LAT>(lane, cy, cz);
-    const RowCopies rcp = row_copies(L, (int)sizeof(ST));
-    const int step_y = (int)gridDim.x % tpp, step_z = (int)gridDim.x / tpp;
-    int ty = (int)blockIdx.x % tpp, tz = (int)blockIdx.x / tpp;
-    Ring ring(0, NOUT);
-    for (int it = blockIdx.x; it < ntiles; it += gridDim.x, ring.step(1, NOUT)) {
-      const int o = ring.s;
-      if (!mbar_wait_or_abort(&ofull[o], ring.pass, limit, &abort_flag)) {
-        if (lane == 0 && !abort_flag) {
-          abort_flag = 1;
-          atomicExch(L.status, 1);
-        }
-        break;
-      }
-      const int y0 = y_first + ty * R, z = z_first + tz, nr = min(R, nyf - ty * R);
-      ty += step_y;
-      tz += step_z;
-      if (ty >= tpp) {
-        ty -= tpp;
-        ++tz;
-      }
-      const unsigned char *ost = stages + kInRegion + o * kOutBytes;
-      if (spitch == L.nxp && plain_tile(rcp, y0, z, nr)) {
-        if (elect_one()) {
-          store_plain_tile<LAT, ST, ODD, PITCH>(rcp, smem_u32(ost), y0, z, nr);
-          bulk_commit();
-          bulk_wait_read_all();
-        }
-      } else if (lane < Q) {
-        store_tile_block<LAT, ST, ODD>(L, ost + lane * PITCH * (int)sizeof(ST), lane, cy, cz, y0, z, nr, spitch);
-        bulk_commit();
-        bulk_wait_read_all();
-      }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&oempty[o]);
-    }
-    bulk_wait_all();
   } else {
     // ---------------- consumer warps
     const long long n = L.n + k;
     // steps since the phi and force references, converted once per launch
     const float dn = (float)(n - L.n_eps), dn_force = (float)(n - L.n_force);
     const int ncr = (L.nx + kChunk - 1) / kChunk;  // chunks per row
-    const bool sr = L.fp16_nearest == 0;
     // small divisions by ncr and the warp count as multiplications (c < 2^8)
     const unsigned inv_ncr = (65535u + ncr) / (unsigned)ncr, inv_k = (65535u + kConsumerWarps) / (unsigned)kConsumerWarps;
     int rot = 0;  // chunks dealt so far, modulo the consumer warps (all warps agree)
-    int j = 0;
-    Ring ring(0, NSTAGE), oring(0, NOUT > 0 ? NOUT : 1);
-    for (int it = blockIdx.x; it < ntiles; it += gridDim.x, ++j, ring.step(1, NSTAGE), oring.step(1, NOUT > 0 ? NOUT : 1)) {
+    Ring ring(0, NSTAGE);
+    for (int it = blockIdx.x; it < ntiles; it += gridDim.x, ring.step(1, NSTAGE)) {
       const int s = ring.s;
       if (!mbar_wait_or_abort(&full[s], ring.pass, limit, &abort_flag)) {
         if (lane == 0 && !abort_flag) {
@@ -1167,45 +1068,27 @@ __global__ void __launch_bounds__((row_consumers_single<MINB, row_pair_lattice<L
         }
         break;
       }
-      unsigned char *ostage = nullptr;
-      if (NOUT > 0) {
-        const int o = oring.s;
-        // the storer has finished reading tile j - NOUT from this output stage
-        if (j >= NOUT && !mbar_wait_or_abort(&oempty[o], oring.pass ^ 1u, limit, &abort_flag)) {
-          if (lane == 0 && !abort_flag) {
-            abort_flag = 1;
-            atomicExch(L.status, 1);
-          }
-          break;
-        }
-        ostage = stages + kInRegion + o * kOutBytes;
-      }
       // the tile's chunks (row t, chunk c of the row), dealt round-robin to
       // the consumer warps across tiles so that every warp gets the same share
       const int nch = tile_nr[s] * ncr;
       const int first = warp - rot + (warp < rot ? kConsumerWarps : 0);
-      const unsigned char *stage = stages + s * kInStride;
+      unsigned char *stage = stages + s * kInStride;
       for (int c = first; c < nch; c += kConsumerWarps) {
         const int t = TILED ? (int)((unsigned)c * inv_ncr >> 16) : 0, xc = c - t * ncr;
-        if constexpr (kPair) {
-          if (sr)
-            update_row_pair<LAT, ODD, WALLS, PITCH, (NOUT > 0), true, TILED>(L, stage, t, ctx[s][t], n, dn, dn_force,
-                                                                             xc * kChunk + 2 * lane, ostage);
-          else
-            update_row_pair<LAT, ODD, WALLS, PITCH, (NOUT > 0), false, TILED>(L, stage, t, ctx[s][t], n, dn, dn_force,
-                                                                              xc * kChunk + 2 * lane, ostage);
-        } else
-          update_row_chunk<LAT, ST, ODD, RED, WALLS, PITCH, RS, (NOUT > 0), TILED>(
-              L, stage, t, ctx[s][t], n, dn, dn_force, xc * kChunk + lane, acc, ostage);
+        // a row without a wall layer beside it takes the periodic code (plain
+        // steps): no per-direction choice of slot (D3Q27 512 x 256 x 256 FP32
+        // with walls on y: 1.28 -> 1.22 ms a step)
+        if (WALLS && !RED && RS == 0 && ctx[s][t].solid == 0)
+          update_row_chunk<LAT, ST, ODD, RED, false, PITCH, RS, false, TILED>(L, stage, t, ctx[s][t], n, dn, dn_force,
+                                                                              xc * kChunk + lane, acc);
+        else
+          update_row_chunk<LAT, ST, ODD, RED, WALLS, PITCH, RS, false, TILED>(L, stage, t, ctx[s][t], n, dn, dn_force,
+                                                                              xc * kChunk + lane, acc);
       }
       rot += nch;
       rot -= (int)((unsigned)rot * inv_k >> 16) * kConsumerWarps;
-      if (NOUT > 0) fence_proxy_async_smem();
       __syncwarp();
-      if (lane == 0) {
-        mbar_arrive(&empty[s]);
-        if (NOUT > 0) mbar_arrive(&ofull[oring.s]);
-      }
+      if (lane == 0) mbar_arrive(&empty[s]);
     }
   }
   __syncthreads();
@@ -1224,7 +1107,7 @@ template <class LAT, class ST, bool W, int P, int MINB, int RS, bool TL>
 cudaError_t launch_row_rs(const LatticeDev *L_dev, bool odd, bool red, bool stat, int k, const StepLaunch &ls,
                           cudaStream_t s) {
   using C = RowCfg<LAT, ST, P, MINB>;
-  constexpr int NS = C::kNSS, NO = C::kNOut;
+  constexpr int NS = C::kNSS;
   // static phi with a larger stage count: the static layout (stat)
   const bool st = stat && C::kNSS > C::kNS;
   const int ns_def = st ? C::kNSS : C::kNS;
@@ -1235,25 +1118,26 @@ cudaError_t launch_row_rs(const LatticeDev *L_dev, bool odd, bool red, bool stat
   const int ns = ls.row_stages >= 2 && ls.row_stages < C::kNS ? ls.row_stages : ns_def;
   const dim3 grid(ls.row_grid);
   const int lay = st ? 1 : 0;
+  cudaError_t e;
   if (RS == 0 && !red && (nc != C::kConsumers || ns != ns_def)) {
-    const dim3 block((nc + kRowProducers + (NO ? 1 : 0)) * 32);
-    const int smem = ns * (st ? C::kInS : C::kIn) + NO * C::kOut;
+    const dim3 block((nc + kRowProducers) * 32);
+    const int smem = ns * (st ? C::kInS : C::kIn);
     if (odd)
-      step_row_kernel<LAT, ST, true, false, W, P, NS, MINB, RS, NO, TL, true><<<grid, block, smem, s>>>(L_dev, k, ns, lay);
+      e = launch_chained(step_row_kernel<LAT, ST, true, false, W, P, NS, MINB, RS, TL, true>, grid, block, smem, s, k > 0, L_dev, k, ns, lay);
     else
-      step_row_kernel<LAT, ST, false, false, W, P, NS, MINB, RS, NO, TL, true><<<grid, block, smem, s>>>(L_dev, k, ns, lay);
-    return cudaGetLastError();
+      e = launch_chained(step_row_kernel<LAT, ST, false, false, W, P, NS, MINB, RS, TL, true>, grid, block, smem, s, k > 0, L_dev, k, ns, lay);
+    return e;
   }
   const dim3 block(C::kThreads);
   const int smem = st ? C::kSmemS : C::kSmem;
   if (odd) {
-    if (red) step_row_kernel<LAT, ST, true, true, W, P, NS, MINB, RS, NO, TL><<<grid, block, smem, s>>>(L_dev, k, ns, lay);
-    else step_row_kernel<LAT, ST, true, false, W, P, NS, MINB, RS, NO, TL><<<grid, block, smem, s>>>(L_dev, k, ns, lay);
+    if (red) e = launch_chained(step_row_kernel<LAT, ST, true, true, W, P, NS, MINB, RS, TL>, grid, block, smem, s, k > 0, L_dev, k, ns, lay);
+    else e = launch_chained(step_row_kernel<LAT, ST, true, false, W, P, NS, MINB, RS, TL>, grid, block, smem, s, k > 0, L_dev, k, ns, lay);
   } else {
-    if (red) step_row_kernel<LAT, ST, false, true, W, P, NS, MINB, RS, NO, TL><<<grid, block, smem, s>>>(L_dev, k, ns, lay);
-    else step_row_kernel<LAT, ST, false, false, W, P, NS, MINB, RS, NO, TL><<<grid, block, smem, s>>>(L_dev, k, ns, lay);
+    if (red) e = launch_chained(step_row_kernel<LAT, ST, false, true, W, P, NS, MINB, RS, TL>, grid, block, smem, s, k > 0, L_dev, k, ns, lay);
+    else e = launch_chained(step_row_kernel<LAT, ST, false, false, W, P, NS, MINB, RS, TL>, grid, block, smem, s, k > 0, L_dev, k, ns, lay);
   }
-  return cudaGetLastError();
+  return e;
 }
 
 // red: bit 0 a check step, bit 1 the step decodes with the shift of the
@@ -1285,7 +1169,7 @@ cudaError_t launch_row_t(const LatticeDev *L_dev, bool odd, int red, int k, cons
 template <class LAT, class ST, bool W, int P, int MINB, bool TL, bool ODD, bool RED, int RS, bool TUNED = false>
 cudaError_t configure_row_one(int smem) {
   using C = RowCfg<LAT, ST, P, MINB>;
-  return cudaFuncSetAttribute(step_row_kernel<LAT, ST, ODD, RED, W, P, C::kNSS, MINB, RS, C::kNOut, TL, TUNED>,
+  return cudaFuncSetAttribute(step_row_kernel<LAT, ST, ODD, RED, W, P, C::kNSS, MINB, RS, TL, TUNED>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
 }
 
@@ -1311,15 +1195,15 @@ int configure_row_v(int &occ, int &nc, int &ns) {
 #undef LBM_CFG
   if (e == cudaSuccess) e = configure_row_one<LAT, ST, W, P, MINB, TL, true, false, 0, true>(smem_max);
   if (e == cudaSuccess) e = configure_row_one<LAT, ST, W, P, MINB, TL, false, false, 0, true>(smem_max);
-  const int threads = (nc + kRowProducers + (C::kNOut ? 1 : 0)) * 32;
-  const int smem = ns * C::kIn + C::kNOut * C::kOut;
+  const int threads = (nc + kRowProducers) * 32;
+  const int smem = ns * C::kIn;
   const bool tuned = nc != C::kConsumers || ns != C::kNS;
   if (e == cudaSuccess)
     e = tuned ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                    &occ, step_row_kernel<LAT, ST, true, false, W, P, C::kNSS, MINB, 0, C::kNOut, TL, true>, threads,
+                    &occ, step_row_kernel<LAT, ST, true, false, W, P, C::kNSS, MINB, 0, TL, true>, threads,
                     smem)
               : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                    &occ, step_row_kernel<LAT, ST, true, false, W, P, C::kNSS, MINB, 0, C::kNOut, TL>, threads, smem);
+                    &occ, step_row_kernel<LAT, ST, true, false, W, P, C::kNSS, MINB, 0, TL>, threads, smem);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return 0;

@@ -1,18 +1,16 @@
-// step_row_d3q27_f16.cu -- D3Q27 instantiations of the row-staged kernel, FP16-shifted
+// step_row_d3q27_f16.cu -- D3Q27 instantiations of the row-staged step, FP16-shifted
 // storage (one file per lattice and storage, compiled in parallel).
-#include "step_row.cuh"
+#include "step_group.cuh"
 
 namespace lbm {
 
-constexpr int kMinBlocks = 1;  // blocks per SM at stage pitch 256
-
 cudaError_t launch_step_row_d3q27_f16(const LatticeDev *L_dev, bool odd, int red, int k, const StepLaunch &ls,
                                      cudaStream_t s) {
-  return launch_row_t<D3Q27, __half, kMinBlocks>(L_dev, odd, red, k, ls, s);
+  return launch_group_t<D3Q27>(L_dev, odd, red, k, ls, s);
 }
 
 int plan_row_d3q27_f16(int nx, int nxp, int ny, int nz, unsigned walls, StepLaunch &ls) {
-  return plan_row_t<D3Q27, __half, kMinBlocks>(nx, nxp, ny, nz, walls, ls);
+  return plan_group_t<D3Q27>(nx, nxp, ny, nz, walls, ls);
 }
 
 }  // namespace lbm

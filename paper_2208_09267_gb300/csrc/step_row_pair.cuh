@@ -17,6 +17,10 @@
 
 #include <cuda_fp16.h>
 
+#ifndef LBM_KEEP
+#define LBM_KEEP 0
+#endif
+
 namespace lbm {
 
 typedef float2 P2;  // the values of cells x and x + 1
@@ -46,6 +50,9 @@ __device__ __forceinline__ float ldh(const __half *p) { return __half2float(*p);
 // b q) with the exact FMA remainder, applied until the remainder is that of
 // the nearest quotient (IBM J. Res. Dev. 34, 1990).  Packed for two cells it
 // takes a third of the instructions of four operator divisions and no branch.
+// Operands within 2^-100 .. 2^100 in magnitude: M0 is a sum of halves (at
+// least 2^-56 in magnitude, or zero, where u is not finite either way) and
+// int phi dV is close to the half sigma beside it.
 __device__ __forceinline__ float rcp_approx(float a) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
@@ -63,14 +70,6 @@ __device__ __forceinline__ P2 quot2(P2 a, P2 b, P2 y) {
   q = fma2(fma2(nb, q, a), y, q);
   return fma2(fma2(nb, q, a), y, q);
 }
-// operands far enough inside the normal range that no step of the above
-// leaves it
-__device__ __forceinline__ bool div2_in_range(P2 a, P2 b) {
-  const float m = fminf(fminf(fabsf(lo(a)), fabsf(hi(a))), fminf(fabsf(lo(b)), fabsf(hi(b))));
-  const float x = fmaxf(fmaxf(fabsf(lo(a)), fabsf(hi(a))), fmaxf(fabsf(lo(b)), fabsf(hi(b))));
-  return m > 0x1p-40f && x < 0x1p40f;
-}
-
 // Store the low (hi = false) or high halves of the two cells' packed
 // results: at the even index x (both cells, one 4-byte store) when the
 // destinations are adjacent, else one by one (the second cell only if it
@@ -88,12 +87,15 @@ __device__ __forceinline__ void st_h2(__half *row, unsigned ha, unsigned hb, boo
 // Update cells xa and xa + 1 (xa even) of one staged row.  A second cell
 // past the end of the row (odd nx) repeats the first one's indices; its
 // results are discarded (the adjacent stores write the row's padding slot).
-template <class LAT, bool ODD, bool WALLS, int PITCH, bool OUTS, bool SR, bool TILED = true>
-__device__ __forceinline__ void update_row_pair(const LatticeDev &L, const unsigned char *stage, int t,
+template <class LAT, bool ODD, bool WALLS, int PITCH, bool INPLACE, bool SR, bool TILED = true>
+__device__ __forceinline__ void update_row_pair(const LatticeDev &L, unsigned char *stage, int t,
                                                 const RowCtx &rc, long long n, float dn, float dn_force,
-                                                int xa, unsigned char *ostage) {
+                                                int xa) {
   using Lay = RowLayout<LAT, __half, ODD, PITCH>;
   constexpr int Q = LAT::Q, D = LAT::D;
+  // keep the shift differences of the decode for the encode?  (else they are
+  // formed again from the staged shifts: fewer registers, more loads)
+  constexpr bool kKeep = LBM_KEEP && Q <= 19;
   const int nx = L.nx;
   if (xa >= nx) return;
   const int sp = TILED ? L.nxp : PITCH, tt = TILED ? t : 0;
@@ -208,14 +210,8 @@ __device__ __forceinline__ void update_row_pair(const LatticeDev &L, const unsig
   nb = fma2(f2s(qa & 2u ? 1.f : 0.f), add2(e_yp, e_ym), nb);
   if (D == 3) nb = fma2(f2s(qa & 4u ? 1.f : 0.f), add2(e_zp, e_zm), nb);
   const P2 I = fma2(f2s(L.qw0f), e_c, mul2(f2s(L.qw1f), nb));
-    P2 rho, invM;  // rho~ = M0 / int phi dV
-  if (div2_in_range(M0, I)) {
-    invM = recip2(M0);
-    rho = quot2(M0, I, recip2(I));
-  } else {  // also NaN
-    rho = f2(lo(M0) / lo(I), hi(M0) / hi(I));
-    invM = f2(1.0f / lo(M0), 1.0f / hi(M0));
-  }
+    const P2 invM = recip2(M0);
+  const P2 rho = quot2(M0, I, recip2(I));  // rho~ = M0 / int phi dV
   const P2 pc2 = mul2(rho, f2s(0.5f / 3.0f));
   P2 F0 = fma2(pc2, sub2(e_xp, e_xm), f2s(L.gf[0]));
   P2 F1 = fma2(pc2, sub2(e_yp, e_ym), f2s(L.gf[1]));
@@ -250,13 +246,13 @@ __device__ __forceinline__ void update_row_pair(const LatticeDev &L, const unsig
   const P2 m3uF_s = mul2(f2s(-cf3 * sc), uF);
   SRng rng_a((unsigned)cell, n), rng_b((unsigned)(cell + 1), n);
   const P2 om1_2 = f2s(om1), sc2 = f2s(sc), msc2 = f2s(-sc);
-  __half *orow = OUTS ? reinterpret_cast<__half *>(ostage) + tt * sp : nullptr;
+  __half *orow = INPLACE ? reinterpret_cast<__half *>(stage) + tt * sp : nullptr;
 
-  // destination row of population i: the output stage's row i, or the
-  // population plane (own slot: plane opp(i) of this row; else plane i of
+  // destination row of population i: the staged block that f_opp(i) came
+  // from, or the population plane (own slot: plane opp(i) of this row; else plane i of
   // row (y + c_iy, z + c_iz))
 #define DST_ROW(i, own)                                                                              \
-  ((OUTS) ? orow + (i) * PITCH                                                                       \
+  ((INPLACE) ? orow + opp_of(i) * PITCH                                                              \
           : ((own) ? pop + opp_of(i) * plane + rc.base[1][1]                                         \
                    : pop + (i) * plane + rc.base[1 + LAT::c((i), 2)][1 + LAT::c((i), 1)]))
 
@@ -305,13 +301,13 @@ __device__ __forceinline__ void update_row_pair(const LatticeDev &L, const unsig
     const bool own_a = OWN_DST(i), own_b = OWN_DST(i + 1);
     if (!own_a) {
       if (!OWN_SRC(i + 1))
-        va = fma2(delta[i + 1], msc2, va);
+        va = fma2(kKeep ? delta[i + 1] : fma2(rho2, LD_H_SHIFT(SIG_ROW(cy, cz), cx), ms_x), msc2, va);
       else
         va = fma2(fma2(f2s(-rho0), LD_H_SHIFT(SIG_ROW(cy, cz), cx), s_x), sc2, va);
     }
     if (!own_b) {
       if (!OWN_SRC(i))
-        vb2 = fma2(delta[i], msc2, vb2);
+        vb2 = fma2(kKeep ? delta[i] : fma2(rho2, LD_H_SHIFT(SIG_ROW(-cy, -cz), -cx), ms_x), msc2, vb2);
       else
         vb2 = fma2(fma2(f2s(-rho0), LD_H_SHIFT(SIG_ROW(-cy, -cz), -cx), s_x), sc2, vb2);
     }
