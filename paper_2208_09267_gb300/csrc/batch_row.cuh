@@ -21,9 +21,9 @@
 // (update_row_chunk), so a member's populations are bit-identical alone and
 // in any batch.
 //
-// Check-step sums are reduced per warp and added into per-member FP64 sums
-// with atomics when the item's member changes (their summation order, not
-// the per-cell values, depends on the schedule).
+// Check-step sums are reduced per warp and tile and added into per-member
+// FP64 sums with atomics (their summation order, not the per-cell values,
+// depends on the schedule).
 #pragma once
 
 #include "step_row.cuh"
@@ -205,9 +205,9 @@ __global__ void __launch_bounds__(BatchRowCfg<LAT, ST, P>::kThreads, MINB)
       if (flags_m & 1) {
         if (lane == 0) mbar_arrive(&full[s]);  // nothing to stage: the phase completes
       } else {
-        if (plain_tile(rcp, y0, z, nr)) {
+        if (plain_tile<P == 256>(rcp, y0, z, nr)) {
           if (elect_one()) {
-            issue_plain_tile<LAT, ST, ODD, P>(rcp, smem_u32(stage), smem_u32(&full[s]), bytes, y0, z, nr, true);
+            issue_plain_tile<LAT, ST, ODD, P, P == 256>(rcp, smem_u32(stage), smem_u32(&full[s]), bytes, y0, z, nr, true);
             bulk_g2s(&descs[s], Lg, (unsigned)kDescBytes, &full[s]);
           }
         } else {
@@ -229,10 +229,6 @@ __global__ void __launch_bounds__(BatchRowCfg<LAT, ST, P>::kThreads, MINB)
     }
   } else {
     // ---------------- consumer warps
-    RedAcc acc;
-#pragma unroll
-    for (int q = 0; q < kRedWidth; ++q) acc.v[q] = 0.0;
-    int red_m = -1;  // member whose check sums acc holds
     int rot = 0;     // chunks dealt so far, modulo the consumer warps (all warps agree)
     RowRuns runs(nitems);
     int j = 0;
@@ -249,12 +245,7 @@ __global__ void __launch_bounds__(BatchRowCfg<LAT, ST, P>::kThreads, MINB)
       if (!(flags & 1)) {
         unsigned char *data = stages + s * kStage;
         const LatticeDev &Lm = descs[s];
-        const int m = ctx[s].member;
         const bool red = REDC && (flags & 4) != 0;
-        if (red && m != red_m) {
-          if (red_m >= 0) flush_member_sums(acc, member_sums + (long long)red_m * kRedWidth);
-          red_m = m;
-        }
         const long long n = Lm.n + k;
         const float dn = ctx[s].dn, dn_force = ctx[s].dn_force;
         // FP16 D2Q9/D3Q19 tiles without a check or a pending shift change
@@ -265,31 +256,50 @@ __global__ void __launch_bounds__(BatchRowCfg<LAT, ST, P>::kThreads, MINB)
         const int ncr = pair ? (Lm.nx + 63) >> 6 : (Lm.nx + 31) >> 5;
         const int nch = ctx[s].nr * ncr;
         const int first = (warp - rot + kConsumerWarps) % kConsumerWarps;
-        for (int c = first; c < nch; c += kConsumerWarps) {
-          const int t = c / ncr, xc = c - t * ncr;
-          if constexpr (kPairOK) {
-            if (pair) {
-              if (Lm.fp16_nearest == 0)
-                update_row_pair<LAT, ODD, WALLS, P, false, true>(Lm, data, t, ctx[s].rc[t], n, dn, dn_force,
-                                                                 (xc << 6) + 2 * lane);
-              else
-                update_row_pair<LAT, ODD, WALLS, P, false, false>(Lm, data, t, ctx[s].rc[t], n, dn, dn_force,
-                                                                  (xc << 6) + 2 * lane);
-              continue;
+        const int ncw = pair ? 64 : 32;
+        if (REDC && red) {
+          // check step of this member: the sums of this warp's chunks go to
+          // the member's at once (kept from tile to tile they would hold 24
+          // registers through every step of a check replay)
+          RedAcc acc;
+#pragma unroll
+          for (int q = 0; q < kRedWidth; ++q) acc.v[q] = 0.0;
+          for (int c = first; c < nch; c += kConsumerWarps) {
+            const int t = c / ncr, xc = c - t * ncr;
+            update_row_chunk<LAT, ST, ODD, REDC, WALLS, P, RS>(Lm, data, t, ctx[s].rc[t], n, dn, dn_force,
+                                                               xc * ncw + lane, acc);
+          }
+          if (first < nch) flush_member_sums(acc, member_sums + (long long)ctx[s].member * kRedWidth);
+        } else {
+          RedAcc none;
+          for (int c = first; c < nch; c += kConsumerWarps) {
+            const int t = c / ncr, xc = c - t * ncr;
+            const RowCtx &rc = ctx[s].rc[t];
+            // (a row without a wall layer beside it takes the periodic code)
+            if constexpr (kPairOK) {
+              if (WALLS && rc.solid != 0) {
+                if (Lm.fp16_nearest == 0)
+                  update_row_pair<LAT, ODD, WALLS, P, false, true>(Lm, data, t, rc, n, dn, dn_force, xc * ncw + 2 * lane);
+                else
+                  update_row_pair<LAT, ODD, WALLS, P, false, false>(Lm, data, t, rc, n, dn, dn_force, xc * ncw + 2 * lane);
+              } else {
+                if (Lm.fp16_nearest == 0)
+                  update_row_pair<LAT, ODD, false, P, false, true>(Lm, data, t, rc, n, dn, dn_force, xc * ncw + 2 * lane);
+                else
+                  update_row_pair<LAT, ODD, false, P, false, false>(Lm, data, t, rc, n, dn, dn_force, xc * ncw + 2 * lane);
+              }
+            } else if (WALLS && RS == 0 && rc.solid == 0) {
+              update_row_chunk<LAT, ST, ODD, false, false, P, RS>(Lm, data, t, rc, n, dn, dn_force, xc * ncw + lane, none);
+            } else {
+              update_row_chunk<LAT, ST, ODD, false, WALLS, P, RS>(Lm, data, t, rc, n, dn, dn_force, xc * ncw + lane, none);
             }
           }
-          const int x = (xc << 5) + lane;
-          if (red)
-            update_row_chunk<LAT, ST, ODD, REDC, WALLS, P, RS>(Lm, data, t, ctx[s].rc[t], n, dn, dn_force, x, acc);
-          else
-            update_row_chunk<LAT, ST, ODD, false, WALLS, P, RS>(Lm, data, t, ctx[s].rc[t], n, dn, dn_force, x, acc);
         }
         rot = (rot + nch) % kConsumerWarps;
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty[s]);
     }
-    if (REDC && red_m >= 0) flush_member_sums(acc, member_sums + (long long)red_m * kRedWidth);
   }
 }
 

@@ -52,30 +52,6 @@ struct GroupCfg {
   static_assert(kNS >= kNG && kNG % kGroupHelpers == 0, "every group needs a stage");
 };
 
-// Bytes the copies of a tile of nr rows bring.
-template <class LAT, bool ODD>
-__device__ __forceinline__ unsigned tile_bytes(int nr, int nxp, bool tv) {
-  constexpr int D = LAT::D;
-  const int rows2 = LAT::Q * nr + (ODD ? (D == 3 ? 3 : 1) * (nr + 2) : nr);          // 2-byte rows
-  const int rows4 = (tv ? 2 : 1) * (nr + 2 + (D == 3 ? 2 * nr : 0));                 // 4-byte rows
-  return (unsigned)(nxp * (2 * rows2 + 4 * rows4));
-}
-
-__device__ __forceinline__ void st_release(int *p, int v) {
-  asm volatile("st.release.cta.shared::cta.s32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
-}
-// Bounded wait until *p reaches v.
-__device__ __forceinline__ bool wait_issued(const int *p, int v, unsigned limit, volatile int *abort) {
-  for (unsigned i = 0; i < limit; ++i) {
-    int have;
-    asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];" : "=r"(have) : "r"(smem_u32(p)) : "memory");
-    if (have >= v) return true;
-    if (*abort) return false;
-    __nanosleep(64);
-  }
-  return false;
-}
-
 // RED: a check step, RS = 1: the step after a phi refresh; both update one
 // cell per lane.
 template <class LAT, bool ODD, bool RED, bool WALLS, int PITCH, int RS, bool TILED>
@@ -149,7 +125,8 @@ __global__ void __launch_bounds__(kGroupThreads, 1)
     const bool producer = ((warp - kGroupConsumers) & 1) == 0;
     const bool withhold = L.withhold_copies != 0;
     const RowCopies rcp = row_copies(L, 2);
-    const bool merge = spitch == nxp;
+    // (tiles of a shorter pitch take the tiled layout: only 512 leaves a choice)
+    const bool merge = TILED || PITCH == 256 || spitch == nxp;
     const CtxLane cl(lane);
     const int stride = kGroupHelpers * (int)gridDim.x, it0 = (int)blockIdx.x + help * (int)gridDim.x;
     const int step_y = stride % tpp, step_z = stride / tpp;
@@ -166,7 +143,7 @@ __global__ void __launch_bounds__(kGroupThreads, 1)
         ty -= tpp;
         ++tz;
       }
-      const bool plain = plain_tile(rcp, y0, z, nr);
+      const bool plain = plain_tile<TILED>(rcp, y0, z, nr);
       if (producer) {
         if (j >= NSTAGE && !mbar_wait_or_abort(&empty[s], ring.pass ^ 1u, limit, &abort_flag)) {
           give_up();
@@ -176,10 +153,10 @@ __global__ void __launch_bounds__(kGroupThreads, 1)
         if (lane == 0) tile_nr[s] = nr;
         __syncwarp();
         if (withhold) continue;
-        const unsigned bytes = tile_bytes<LAT, ODD>(nr, nxp, rcp.deps != nullptr);
+        const unsigned bytes = tile_bytes<LAT, __half, ODD>(nr, nxp, rcp.deps != nullptr);
         if (plain) {
           if (elect_one())
-            issue_plain_tile<LAT, __half, ODD, PITCH>(rcp, smem_u32(stage), smem_u32(&full[s]), bytes, y0, z, nr, merge);
+            issue_plain_tile<LAT, __half, ODD, PITCH, TILED>(rcp, smem_u32(stage), smem_u32(&full[s]), bytes, y0, z, nr, merge);
         } else {
           if (lane == 0) mbar_arrive_expect_tx(&full[s], bytes);
           __syncwarp();
@@ -196,7 +173,7 @@ __global__ void __launch_bounds__(kGroupThreads, 1)
           break;
         }
         if (plain) {
-          if (elect_one()) store_plain_tile<LAT, __half, ODD, PITCH>(rcp, smem_u32(stage), y0, z, nr);
+          if (elect_one()) store_plain_tile<LAT, __half, ODD, PITCH, TILED>(rcp, smem_u32(stage), y0, z, nr);
         } else if (lane < LAT::Q) {
           const TileCopy c = make_tile_copy<LAT, __half, ODD, PITCH>(L, lane);
           issue_tile_copy<true>(c, stage, nullptr, y0, z, nr, ny, nz, nxp, rcp.walls, spitch);

@@ -96,6 +96,21 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned by
       : "memory");
 }
 
+__device__ __forceinline__ void st_release(int *p, int v) {
+  asm volatile("st.release.cta.shared::cta.s32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
+}
+// Bounded wait until *p reaches v.
+__device__ __forceinline__ bool wait_issued(const int *p, int v, unsigned limit, volatile int *abort) {
+  for (unsigned i = 0; i < limit; ++i) {
+    int have;
+    asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];" : "=r"(have) : "r"(smem_u32(p)) : "memory");
+    if (have >= v) return true;
+    if (*abort) return false;
+    __nanosleep(64);
+  }
+  return false;
+}
+
 // Bulk copy of `bytes` from shared to global memory (both 16-byte aligned, a
 // multiple of 16 bytes), tracked in this thread's bulk async-group.
 __device__ __forceinline__ void bulk_s2g(void *dst, const void *src, unsigned bytes) {
@@ -374,21 +389,32 @@ __device__ __forceinline__ RowCopies row_copies(const LatticeDev &L, int esize) 
   return c;
 }
 
-// Do the rows y0 - 1 .. y0 + nr lie inside the plane, with no wall layer next
-// to the tile?  Then every block of the tile is one run of rows (planes
-// z - 1 and z + 1 may wrap around) and the one-lane loops below apply.
+// No wall layer next to the tile?  Then its rows are runs of the plane (planes
+// z - 1 and z + 1 may wrap around; rows y0 - 1 and y0 + nr too with WRAP) and
+// the one-lane loops below apply.  WRAP is for tiles of several rows, where
+// the tiles at the y ends are many (an eighth at 64^3): taking those through
+// the lane-parallel path made a 64^3 FP16 step 14.5 us instead of 9.5, a 61 x
+// 75 x 67 FP32 one 15.2 instead of 11.2.  With rows of 256 cells they are 2 in
+// 256 and the extra code costs more (FP16 256^3: 287 -> 300 us a step).
+template <bool WRAP>
 __device__ __forceinline__ bool plain_tile(const RowCopies &c, int y0, int z, int nr) {
-  const int m = (c.walls & 2u) ? 2 : 1;
-  if (y0 < m || y0 + nr > c.ny - m) return false;
+  if (!WRAP && (y0 < 1 || y0 + nr >= c.ny)) return false;
+  if ((c.walls & 2u) && (y0 < 2 || y0 + nr > c.ny - 2)) return false;
   return !(c.walls & 4u) || (z >= 2 && z < c.nz - 2);
 }
+
+// Does a tile without walls beside it wrap around in y?
+__device__ __forceinline__ bool edge_tile(const RowCopies &c, int y0, int nr) { return y0 == 0 || y0 + nr == c.ny; }
 
 // Stage a plain tile: one lane issues the copies of every block in a row,
 // unrolled over compile-time directions.  With the blocks spread over the
 // lanes instead, each copy is issued on its own all the same (its operands
 // are uniform registers), after some 20 instructions that pick the lane.
-template <class LAT, class ST, bool ODD, int PITCH>
-__device__ __forceinline__ void issue_plain_tile(const RowCopies &c, unsigned stage, unsigned bar, unsigned bytes,
+// EDGE: the rows beside the tile wrap around in y (code of its own: the tests
+// of every copy, put into the straight line of the other tiles, made a 256^3
+// FP16 step 385 us).
+template <class LAT, class ST, bool ODD, int PITCH, bool EDGE>
+__device__ __forceinline__ void issue_plain_copies(const RowCopies &c, unsigned stage, unsigned bar, unsigned bytes,
                                                  int y0, int z, int nr, bool merge) {
   using Lay = RowLayout<LAT, ST, ODD, PITCH>;
   constexpr int D = LAT::D;
@@ -397,13 +423,34 @@ __device__ __forceinline__ void issue_plain_tile(const RowCopies &c, unsigned st
                  "l"(src), "r"(n), "r"(bar)
                  : "memory");
   };
-  // n rows of a field from byte offset off, landing at slots of PITCH elements
-  // when the stored pitch differs (one-row tiles: blocks of up to 3 rows)
-  auto rows = [&](unsigned dst, const char *src, int n, unsigned row_bytes, unsigned slot_bytes) {
+  // does row y0 - 1, or y0 + nr, wrap around?
+  const bool lo = EDGE && y0 == 0, hi = EDGE && y0 + nr == c.ny;
+  // n rows from src; the first, or the last, of them wraps around
+  auto run = [&](unsigned dst, const char *src, int n, unsigned row_bytes, bool first, bool last) {
+    const unsigned span = (unsigned)c.ny * row_bytes;
+    if (first) {
+      copy(dst, src + span, row_bytes);
+      dst += row_bytes;
+      src += row_bytes;
+      --n;
+    }
+    if (last) {
+      --n;
+      copy(dst + n * row_bytes, src + (long long)n * row_bytes - span, row_bytes);
+    }
+    if (n > 0) copy(dst, src, (unsigned)n * row_bytes);
+  };
+  // rows y0 - 1 .. y0 + nr of a field from the first of them on, landing at
+  // slots of PITCH elements when the stored pitch differs (one-row tiles)
+  auto rows = [&](unsigned dst, const char *src, unsigned row_bytes, unsigned slot_bytes) {
     if (merge) {
-      copy(dst, src, (unsigned)n * row_bytes);
+      if (lo || hi) run(dst, src, nr + 2, row_bytes, lo, hi);
+      else copy(dst, src, (unsigned)(nr + 2) * row_bytes);
     } else {
-      for (int k = 0; k < n; ++k) copy(dst + k * slot_bytes, src + k * row_bytes, row_bytes);
+      const unsigned span = (unsigned)c.ny * row_bytes;
+      copy(dst, lo ? src + span : src, row_bytes);
+      copy(dst + slot_bytes, src + row_bytes, row_bytes);
+      copy(dst + 2 * slot_bytes, hi ? src + 2 * row_bytes - span : src + 2 * row_bytes, row_bytes);
     }
   };
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
@@ -423,16 +470,17 @@ __device__ __forceinline__ void issue_plain_tile(const RowCopies &c, unsigned st
     if (cz < 0) p += ozp;
     if (cy > 0) p -= pb;
     if (cy < 0) p += pb;
-    copy(stage + i * Lay::kPopBytes, p, (unsigned)nr * pb);
+    if ((cy > 0 && lo) || (cy < 0 && hi)) run(stage + i * Lay::kPopBytes, p, nr, pb, cy > 0, cy < 0);
+    else copy(stage + i * Lay::kPopBytes, p, (unsigned)nr * pb);
     src += c.plane_bytes;
   }
   const unsigned sb = (unsigned)c.nxp * 2u, fb = (unsigned)c.nxp * 4u;
   const char *sg = c.sig + (long long)r0 * sb;
   if (ODD) {
-    rows(stage + Lay::kSigOff + (D == 3 ? 3 * Lay::kSigBytes : 0), sg - sb, nr + 2, sb, Lay::kSigBytes);
+    rows(stage + Lay::kSigOff + (D == 3 ? 3 * Lay::kSigBytes : 0), sg - sb, sb, Lay::kSigBytes);
     if (D == 3) {
-      rows(stage + Lay::kSigOff, sg + (long long)dzm * sb - sb, nr + 2, sb, Lay::kSigBytes);
-      rows(stage + Lay::kSigOff + 6 * Lay::kSigBytes, sg + (long long)dzp * sb - sb, nr + 2, sb, Lay::kSigBytes);
+      rows(stage + Lay::kSigOff, sg + (long long)dzm * sb - sb, sb, Lay::kSigBytes);
+      rows(stage + Lay::kSigOff + 6 * Lay::kSigBytes, sg + (long long)dzp * sb - sb, sb, Lay::kSigBytes);
     }
   } else {
     copy(stage + Lay::kSigOff, sg, (unsigned)nr * sb);
@@ -443,7 +491,7 @@ __device__ __forceinline__ void issue_plain_tile(const RowCopies &c, unsigned st
     if (f == 1 && !c.deps) break;
     const char *fld = (f == 0 ? c.eps : c.deps) + fo;
     const unsigned off = stage + (f == 0 ? Lay::kEpsOff : Lay::kDepsOff);
-    rows(off, fld - fb, nr + 2, fb, Lay::kRowBytes);
+    rows(off, fld - fb, fb, Lay::kRowBytes);
     if (D == 3) {
       copy(off + 3 * Lay::kRowBytes, fld + fzm, (unsigned)nr * fb);
       copy(off + 4 * Lay::kRowBytes, fld + fzp, (unsigned)nr * fb);
@@ -451,16 +499,29 @@ __device__ __forceinline__ void issue_plain_tile(const RowCopies &c, unsigned st
   }
 }
 
+template <class LAT, class ST, bool ODD, int PITCH, bool WRAP>
+__device__ __forceinline__ void issue_plain_tile(const RowCopies &c, unsigned stage, unsigned bar, unsigned bytes,
+                                                 int y0, int z, int nr, bool merge) {
+  if (WRAP && edge_tile(c, y0, nr))
+    issue_plain_copies<LAT, ST, ODD, PITCH, true>(c, stage, bar, bytes, y0, z, nr, merge);
+  else
+    issue_plain_copies<LAT, ST, ODD, PITCH, false>(c, stage, bar, bytes, y0, z, nr, merge);
+}
+
 // Store a plain tile's population blocks back to where issue_plain_tile
 // loaded them from.
-template <class LAT, class ST, bool ODD, int PITCH>
-__device__ __forceinline__ void store_plain_tile(const RowCopies &c, unsigned stage, int y0, int z, int nr) {
+template <class LAT, class ST, bool ODD, int PITCH, bool EDGE>
+__device__ __forceinline__ void store_plain_copies(const RowCopies &c, unsigned stage, int y0, int z, int nr) {
   using Lay = RowLayout<LAT, ST, ODD, PITCH>;
   constexpr int D = LAT::D;
   const int dzm = D == 3 ? (z == 0 ? c.nz - 1 : -1) * c.ny : 0, dzp = D == 3 ? (z == c.nz - 1 ? 1 - c.nz : 1) * c.ny : 0;
   const unsigned pb = (unsigned)(c.nxp * (int)sizeof(ST));
   const long long ozm = (long long)dzm * pb, ozp = (long long)dzp * pb;
   char *dst = const_cast<char *>(c.pop) + (long long)(z * c.ny + y0) * pb;
+  const bool lo = EDGE && y0 == 0, hi = EDGE && y0 + nr == c.ny;
+  auto copy = [&](char *p, unsigned from, unsigned n) {
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(p), "r"(from), "r"(n) : "memory");
+  };
 #pragma unroll
   for (int j = 0; j < LAT::Q; ++j) {
     const int i = ODD ? opp_of(j) : j;
@@ -470,11 +531,37 @@ __device__ __forceinline__ void store_plain_tile(const RowCopies &c, unsigned st
     if (cz < 0) p += ozp;
     if (cy > 0) p -= pb;
     if (cy < 0) p += pb;
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(p), "r"(stage + i * Lay::kPopBytes),
-                 "r"((unsigned)nr * pb)
-                 : "memory");
+    unsigned from = stage + i * Lay::kPopBytes;
+    int n = nr;
+    if (cy > 0 && lo) {  // the first row wraps around
+      copy(p + (unsigned)c.ny * pb, from, pb);
+      p += pb;
+      from += pb;
+      --n;
+    }
+    if (cy < 0 && hi) {  // the last one does
+      --n;
+      copy(p + (long long)n * pb - (unsigned)c.ny * pb, from + n * pb, pb);
+    }
+    if (n > 0) copy(p, from, (unsigned)n * pb);
     dst += c.plane_bytes;
   }
+}
+
+template <class LAT, class ST, bool ODD, int PITCH, bool WRAP>
+__device__ __forceinline__ void store_plain_tile(const RowCopies &c, unsigned stage, int y0, int z, int nr) {
+  if (WRAP && edge_tile(c, y0, nr)) store_plain_copies<LAT, ST, ODD, PITCH, true>(c, stage, y0, z, nr);
+  else store_plain_copies<LAT, ST, ODD, PITCH, false>(c, stage, y0, z, nr);
+}
+
+// Bytes the copies of a tile of nr rows bring.
+template <class LAT, class ST, bool ODD>
+__device__ __forceinline__ unsigned tile_bytes(int nr, int nxp, bool tv) {
+  constexpr int D = LAT::D;
+  const int pops = LAT::Q * (int)sizeof(ST) * nr;
+  const int shifts = 2 * (ODD ? (D == 3 ? 3 : 1) * (nr + 2) : nr);
+  const int phis = 4 * (tv ? 2 : 1) * (nr + 2 + (D == 3 ? 2 * nr : 0));
+  return (unsigned)(nxp * (pops + shifts + phis));
 }
 
 // The row contexts of a tile, written by the producer warp (lanes in
@@ -1001,7 +1088,8 @@ __global__ void __launch_bounds__((row_consumers_single<MINB>() + kRowProducers)
     int ty = it0 % tpp, tz = it0 / tpp;
     const RowCopies rcp = row_copies(L, (int)sizeof(ST));
     const CtxLane cl(lane);
-    const bool merge = spitch == nxp;
+    // (tiles of a shorter pitch take the tiled layout: only 512 leaves a choice)
+    const bool merge = TILED || PITCH == 256 || spitch == nxp;
     int issued_upto = -1;  // last tile index j whose copies this warp issued
     int j = pw;
     Ring ring(pw, NSTAGE);  // tile j's stage and pass, carried along
@@ -1030,9 +1118,9 @@ __global__ void __launch_bounds__((row_consumers_single<MINB>() + kRowProducers)
       __syncwarp();
       if (!withhold) {
         unsigned char *stage = stages + s * kInStride;
-        if (plain_tile(rcp, y0, z, nr)) {
+        if (plain_tile<TILED>(rcp, y0, z, nr)) {
           if (elect_one())
-            issue_plain_tile<LAT, ST, ODD, PITCH>(rcp, smem_u32(stage), smem_u32(&full[s]), bytes, y0, z, nr, merge);
+            issue_plain_tile<LAT, ST, ODD, PITCH, TILED>(rcp, smem_u32(stage), smem_u32(&full[s]), bytes, y0, z, nr, merge);
         } else {
           if (lane == 0) mbar_arrive_expect_tx(&full[s], bytes);
           __syncwarp();
