@@ -52,15 +52,14 @@ struct GroupCfg {
   static_assert(kNS >= kNG && kNG % kGroupHelpers == 0, "every group needs a stage");
 };
 
-// RED: a check step, RS = 1: the step after a phi refresh; both update one
-// cell per lane.
+// RED: a check step (one cell per lane), RS = 1: the step after a phi refresh.
 template <class LAT, bool ODD, bool RED, bool WALLS, int PITCH, int RS, bool TILED>
 __global__ void __launch_bounds__(kGroupThreads, 1)
     step_group_kernel(const LatticeDev *__restrict__ Lp, int k, int lay_static) {
   using Lay = RowLayout<LAT, __half, ODD, PITCH>;
   using Cfg = GroupCfg<LAT, PITCH>;
   constexpr int kMaxStage = Cfg::kNSS;
-  constexpr bool kPair = !RED && RS == 0;
+  constexpr bool kPair = !RED;
   const int NSTAGE = lay_static ? Cfg::kNSS : Cfg::kNS;
   const int kInStride = lay_static ? Lay::kDepsOff : Lay::kStageBytes;
   __shared__ LatticeDev Ls;
@@ -229,7 +228,7 @@ __global__ void __launch_bounds__(kGroupThreads, 1)
         const bool at_wall = WALLS && __any_sync(__activemask(), rc.solid != 0);
         if constexpr (kPair) {
           auto go = [&](auto walls_c, auto sr_c) {
-            update_row_pair<LAT, ODD, decltype(walls_c)::value, PITCH, true, decltype(sr_c)::value, TILED>(
+            update_row_pair<LAT, ODD, decltype(walls_c)::value, PITCH, true, decltype(sr_c)::value, TILED, RS != 0>(
                 L, stage, t, rc, n, dn, dn_force, x);
           };
           if (WALLS && at_wall) {

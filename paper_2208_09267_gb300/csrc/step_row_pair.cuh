@@ -1,6 +1,5 @@
 // step_row_pair.cuh -- the row kernel's per-cell update for two adjacent
-// cells per lane, FP16-shifted storage, plain steps (no check sums, no
-// pending shift change).
+// cells per lane, FP16-shifted storage, plain steps (no check sums).
 //
 // Each operation of update_row_chunk is applied to the cells x and x + 1 at
 // once as a packed FP32 pair operation (fma/add/mul .rn.f32x2: per
@@ -16,10 +15,6 @@
 #pragma once
 
 #include <cuda_fp16.h>
-
-#ifndef LBM_KEEP
-#define LBM_KEEP 0
-#endif
 
 namespace lbm {
 
@@ -84,18 +79,18 @@ __device__ __forceinline__ void st_h2(__half *row, unsigned ha, unsigned hb, boo
   }
 }
 
+// RESHIFT: the step after a phi refresh (decode with the old shift, encode
+// with the new one); as a one-cell update it took 0.45 ms of a refresh interval
+// of ten 256^3 steps at 0.28.
 // Update cells xa and xa + 1 (xa even) of one staged row.  A second cell
 // past the end of the row (odd nx) repeats the first one's indices; its
 // results are discarded (the adjacent stores write the row's padding slot).
-template <class LAT, bool ODD, bool WALLS, int PITCH, bool INPLACE, bool SR, bool TILED = true>
+template <class LAT, bool ODD, bool WALLS, int PITCH, bool INPLACE, bool SR, bool TILED = true, bool RESHIFT = false>
 __device__ __forceinline__ void update_row_pair(const LatticeDev &L, unsigned char *stage, int t,
                                                 const RowCtx &rc, long long n, float dn, float dn_force,
                                                 int xa) {
   using Lay = RowLayout<LAT, __half, ODD, PITCH>;
   constexpr int Q = LAT::Q, D = LAT::D;
-  // keep the shift differences of the decode for the encode?  (else they are
-  // formed again from the staged shifts: fewer registers, more loads)
-  constexpr bool kKeep = LBM_KEEP && Q <= 19;
   const int nx = L.nx;
   if (xa >= nx) return;
   const int sp = TILED ? L.nxp : PITCH, tt = TILED ? t : 0;
@@ -131,24 +126,23 @@ __device__ __forceinline__ void update_row_pair(const LatticeDev &L, unsigned ch
 #define OWN_DST(i) (!ODD || (i) == 0 || (WALLS && ((rc.solid >> ((1 + LAT::c((i), 2)) * 3 + (1 + LAT::c((i), 1)))) & 1u)))
 
   const P2 sig_own = ld_h2(SIG_ROW(0, 0) + xa);
-  const P2 s_x = mul2(f2s(rho0), sig_own);
+  const __half *__restrict__ srd = L.sig_rd;
+  const P2 s_x = mul2(f2s(rho0), RESHIFT ? ld_h2(srd + cell) : sig_own);
   const P2 ms_x = f2(-lo(s_x), -hi(s_x));
   const P2 rho2 = f2s(rho0), scale2 = f2s(scale);
 
   // 1. decode (update_row_chunk step 1, in storage units)
-  P2 d[Q], delta[Q];
+  P2 d[Q];
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
     const int cx = LAT::c(i, 0), cy = LAT::c(i, 1), cz = LAT::c(i, 2);
     const __half *pr = prow + i * PITCH;
     if (OWN_SRC(i)) {
-      delta[i] = f2s(0.f);
       d[i] = ld_h2(pr + xa);
     } else {
       const P2 q = LD_H_SHIFT(pr, -cx);
-      const P2 sw = LD_H_SHIFT(SIG_ROW(-cy, -cz), -cx);
-      delta[i] = fma2(rho2, sw, ms_x);
-      d[i] = fma2(delta[i], scale2, q);
+      const P2 sw = RESHIFT ? LD_H_SHIFT(srd + rc.base[1 - cz][1 - cy], -cx) : LD_H_SHIFT(SIG_ROW(-cy, -cz), -cx);
+      d[i] = fma2(fma2(rho2, sw, ms_x), scale2, q);
     }
   }
 
@@ -251,6 +245,7 @@ __device__ __forceinline__ void update_row_pair(const LatticeDev &L, unsigned ch
   // destination row of population i: the staged block that f_opp(i) came
   // from, or the population plane (own slot: plane opp(i) of this row; else plane i of
   // row (y + c_iy, z + c_iz))
+  const P2 enc_own = RESHIFT ? fma2(f2s(-rho0), sig_own, s_x) : f2s(0.f);
 #define DST_ROW(i, own)                                                                              \
   ((INPLACE) ? orow + opp_of(i) * PITCH                                                              \
           : ((own) ? pop + opp_of(i) * plane + rc.base[1][1]                                         \
@@ -258,7 +253,8 @@ __device__ __forceinline__ void update_row_pair(const LatticeDev &L, unsigned ch
 
   {
     // rest population
-    const P2 v = fma2(om1_2, d[0], fma2(f2s(omega_s), fma2(M0, m15usq, dM), m3uF_s));
+    P2 v = fma2(om1_2, d[0], fma2(f2s(omega_s), fma2(M0, m15usq, dM), m3uF_s));
+    if (RESHIFT) v = fma2(enc_own, sc2, v);
     __half ha, hb;
     if (SR) {
       ha = half_sr(lo(v), rng_a.next13());
@@ -297,17 +293,21 @@ __device__ __forceinline__ void update_row_pair(const LatticeDev &L, unsigned ch
     P2 va = fma2(om1_2, d[i], add2(A, B));
     P2 vb2 = fma2(om1_2, d[i + 1], sub2(A, B));
     // encode against the shift of the storage cell (update_row_chunk's
-    // ENCODE_POP without a pending shift change)
+    // ENCODE_POP).  The shift differences are formed again, not kept from the
+    // decode: 36 registers against a load and two conversions each, and 96
+    // registers a thread give a third more warps.
     const bool own_a = OWN_DST(i), own_b = OWN_DST(i + 1);
+    if (RESHIFT && own_a) va = fma2(enc_own, sc2, va);
+    if (RESHIFT && own_b) vb2 = fma2(enc_own, sc2, vb2);
     if (!own_a) {
-      if (!OWN_SRC(i + 1))
-        va = fma2(kKeep ? delta[i + 1] : fma2(rho2, LD_H_SHIFT(SIG_ROW(cy, cz), cx), ms_x), msc2, va);
+      if (!RESHIFT && !OWN_SRC(i + 1))
+        va = fma2(fma2(rho2, LD_H_SHIFT(SIG_ROW(cy, cz), cx), ms_x), msc2, va);
       else
         va = fma2(fma2(f2s(-rho0), LD_H_SHIFT(SIG_ROW(cy, cz), cx), s_x), sc2, va);
     }
     if (!own_b) {
-      if (!OWN_SRC(i))
-        vb2 = fma2(kKeep ? delta[i] : fma2(rho2, LD_H_SHIFT(SIG_ROW(-cy, -cz), -cx), ms_x), msc2, vb2);
+      if (!RESHIFT && !OWN_SRC(i))
+        vb2 = fma2(fma2(rho2, LD_H_SHIFT(SIG_ROW(-cy, -cz), -cx), ms_x), msc2, vb2);
       else
         vb2 = fma2(fma2(f2s(-rho0), LD_H_SHIFT(SIG_ROW(-cy, -cz), -cx), s_x), sc2, vb2);
     }

@@ -45,3 +45,28 @@ def test_plain_steps_equal_check_steps(lattice, shape, walls, deps, rounding):
         out.append(lat.populations())
         lat.close()
     assert np.array_equal(*out)
+
+
+@pytest.mark.parametrize("lattice,shape,walls", [
+    ("D2Q9", (13, 40, 1), 2), ("D3Q19", (75, 11, 9), 2), ("D3Q19", (256, 9, 8), 0), ("D3Q27", (300, 6, 7), 0),
+    ("D3Q27", (33, 8, 6), 4)])
+def test_the_step_after_a_refresh_equals_its_check_step(lattice, shape, walls):
+    """Decoding with the old shift and encoding with the new one, two cells per
+    lane, at an even and at an odd step."""
+    n = int(np.prod(shape))
+    rng = np.random.default_rng(n + 1)
+    phis = [(0.5 + 0.4 * rng.random(n)).astype(np.float32) for _ in range(3)]
+    out = []
+    for check in (False, True):
+        lat = lbm.Lattice(lattice, shape, tau=0.6, storage="fp16", walls=walls, kernel="row")
+        lat.set_epsilon(phis[0])
+        lat.set_force((1e-5, -3e-6, 2e-6))
+        lat.init_equilibrium()
+        lat.step(4)
+        for phi in phis[1:]:                  # refreshed before step 4 and step 7
+            lat.set_epsilon(phi, n_ref=lat.steps_done)
+            for _ in range(3):
+                lat.step(1, check_every=0 if check else -1)
+        out.append(lat.populations())
+        lat.close()
+    assert np.array_equal(*out)
