@@ -58,7 +58,7 @@ StepLaunch make_launch(int nx, int ny, int nz, int bx, int by) {
   ls.row = 0;
   ls.row_grid = 0;
   ls.row_smem_even = ls.row_smem_odd = 0;
-  ls.row_consumers = ls.row_stages = 0;
+  ls.row_consumers = ls.row_stages = ls.exact_split = 0;
   return ls;
 }
 
@@ -75,6 +75,7 @@ StepLaunch make_launch_exact(int nx, int ny, int nz, int bx, int by) {
     int t = 256;
     while (t > 32 && (cells + t - 1) / t < 8LL * 152) t /= 2;
     ls.block = dim3(t, 1, 1);
+    ls.exact_split = t == 32 && cells <= 304LL * 32;  // see step_exact_split_kernel
   }
   ls.block_threads = (int)(ls.block.x * ls.block.y);
   ls.grid = dim3((unsigned)((cells + ls.block_threads - 1) / ls.block_threads), 1, 1);
@@ -152,17 +153,17 @@ cudaError_t launch_finalize(const double *partials, int nblocks, double *out, cu
 // times per cell (own row, z-1, z+1) instead of seven; x neighbours come
 // from the row the warp has just read (L1).  Same sum order as eq. (quad)
 // is written everywhere: x pair, y pair, z pair.
-constexpr int kShiftSeg = 32;  // rows of y per thread
+constexpr int kShiftSeg = 32;  // most rows of y per thread
 
 __global__ void shift_kernel(const float *eps, __half *sig, int nx, int nxp, int ny, int nz, unsigned qa,
-                             float w0, float w1) {
+                             float w0, float w1, int seg) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= nxp) return;
-  const int nseg = (ny + kShiftSeg - 1) / kShiftSeg;
+  const int nseg = (ny + seg - 1) / seg;
   const long long plane = (long long)ny * nxp;
   for (long long t = blockIdx.y; t < (long long)nz * nseg; t += gridDim.y) {
-    const int z = (int)(t / nseg), y0 = (int)(t % nseg) * kShiftSeg;
-    const int y1 = y0 + kShiftSeg < ny ? y0 + kShiftSeg : ny;
+    const int z = (int)(t / nseg), y0 = (int)(t % nseg) * seg;
+    const int y1 = y0 + seg < ny ? y0 + seg : ny;
     const long long pz = (long long)z * plane;
     if (x >= nx) {  // row padding: a valid value that nothing decodes
       for (int y = y0; y < y1; ++y) sig[pz + (long long)y * nxp + x] = __float2half_rn(1.0f);
@@ -189,10 +190,15 @@ __global__ void shift_kernel(const float *eps, __half *sig, int nx, int nxp, int
 
 cudaError_t launch_shift(const LatticeDev &h, const float *eps, __half *sig, cudaStream_t s) {
   const int block = h.nxp >= 256 ? 256 : (h.nxp >= 128 ? 128 : 64);
-  const long long work = (long long)h.nz * ((h.ny + kShiftSeg - 1) / kShiftSeg);
+  // shorter walks where the lattice is too small to fill the chip with long
+  // ones (each row of a walk waits for its loads: a walk of 32 rows takes 17
+  // to 20 us, on a 64^2 lattice too)
+  int seg = kShiftSeg;
+  while (seg > 2 && (long long)h.nxp * h.nz * ((h.ny + seg - 1) / seg) < 152LL * 2048) seg /= 2;
+  const long long work = (long long)h.nz * ((h.ny + seg - 1) / seg);
   const dim3 grid((unsigned)((h.nxp + block - 1) / block), (unsigned)(work < 65535 ? work : 65535));
   shift_kernel<<<grid, block, 0, s>>>(eps, sig, h.nx, h.nxp, h.ny, h.nz, h.quad_axes, (float)h.qw0,
-                                      (float)h.qw1);
+                                      (float)h.qw1, seg);
   return cudaGetLastError();
 }
 

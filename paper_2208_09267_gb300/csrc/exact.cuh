@@ -132,38 +132,45 @@ __device__ __forceinline__ double dot_c(int i, const double *v) {
   return s;
 }
 
-// M0 and J in ascending i
+// M0, and the momentum along axis a, in ascending i
 template <class LAT>
-__device__ __forceinline__ void sums_exact(const double *f, MacroD &m) {
-  constexpr int Q = LAT::Q, D = LAT::D;
-  m.M0 = f[0];
+__device__ __forceinline__ double sum_m0(const double *f) {
+  double s = f[0];
 #pragma unroll
-  for (int i = 1; i < Q; ++i) m.M0 = m.M0 + f[i];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    m.J[a] = 0.0;
-    if (a >= D) continue;
-    bool any = false;
-#pragma unroll
-    for (int i = 1; i < Q; ++i) {
-      if (LAT::c(i, a) == 0) continue;
-      const double t = LAT::c(i, a) > 0 ? f[i] : -f[i];
-      m.J[a] = any ? m.J[a] + t : t;
-      any = true;
-    }
-  }
+  for (int i = 1; i < LAT::Q; ++i) s = s + f[i];
+  return s;
 }
 
-// rho~, F and u from M0 and J; DRAG: the lattice may carry the drag law
-template <class LAT, bool F64, bool DRAG>
-__device__ __forceinline__ void macro_from_sums(const LatticeDev &L, long long n, const Coords &C, MacroD &m) {
-  constexpr int D = LAT::D;
+template <class LAT>
+__device__ __forceinline__ double sum_j(const double *f, int a) {
+  double s = 0.0;
+  bool any = false;
+#pragma unroll
+  for (int i = 1; i < LAT::Q; ++i) {
+    if (LAT::c(i, a) == 0) continue;
+    const double t = LAT::c(i, a) > 0 ? f[i] : -f[i];
+    s = any ? s + t : t;
+    any = true;
+  }
+  return s;
+}
+
+template <class LAT>
+__device__ __forceinline__ void sums_exact(const double *f, MacroD &m) {
+  m.M0 = sum_m0<LAT>(f);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) m.J[a] = a < LAT::D ? sum_j<LAT>(f, a) : 0.0;
+}
+
+// phi at time n on the cell and its face neighbours
+template <class LAT, bool F64>
+__device__ __forceinline__ void phi_stencil(const LatticeDev &L, long long n, const Coords &C, double &e_c,
+                                            double *e_p, double *e_m) {
   const double dn = (double)(n - L.n_eps);
-  const double e_c = eps_at<F64>(L, C.at(0, 0, 0), dn);
-  double e_p[3], e_m[3];
+  e_c = eps_at<F64>(L, C.at(0, 0, 0), dn);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    if (a < D) {
+    if (a < LAT::D) {
       e_p[a] = eps_at<F64>(L, C.at(a == 0, a == 1, a == 2), dn);
       e_m[a] = eps_at<F64>(L, C.at(-(a == 0), -(a == 1), -(a == 2)), dn);
     } else {
@@ -171,6 +178,10 @@ __device__ __forceinline__ void macro_from_sums(const LatticeDev &L, long long n
       e_m[a] = e_c;
     }
   }
+}
+
+// eq. (quad)
+__device__ __forceinline__ double quad_exact(const LatticeDev &L, double e_c, const double *e_p, const double *e_m) {
   double nb = 0.0;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -179,20 +190,30 @@ __device__ __forceinline__ void macro_from_sums(const LatticeDev &L, long long n
       nb = nb + e_m[a];
     }
   }
-  m.I = L.qw0 * e_c + L.qw1 * nb;
-  m.rho = m.M0 / m.I;
-  const double pc = m.rho / 3.0;
+  return L.qw0 * e_c + L.qw1 * nb;
+}
+
+// force along axis a
+template <bool F64>
+__device__ __forceinline__ double force_exact(const LatticeDev &L, long long n, const Coords &C, int a, double rho,
+                                              double e_p, double e_m) {
+  const double pc = rho / 3.0;
   const double hpc = 0.5 * pc;  // pc (0.5 (e_p - e_m)) = (0.5 pc) (e_p - e_m) exactly
-  const double dnf = (double)(n - L.n_force);
-  const long long k = C.at(0, 0, 0);
+  double fext = L.g[a];
+  if (L.has_force) fext = fext + force_at<F64>(L, a, C.at(0, 0, 0), (double)(n - L.n_force));
+  return fext + hpc * (e_p - e_m);
+}
+
+// rho~, F and u from M0 and J; DRAG: the lattice may carry the drag law
+template <class LAT, bool F64, bool DRAG>
+__device__ __forceinline__ void macro_from_sums(const LatticeDev &L, long long n, const Coords &C, MacroD &m) {
+  constexpr int D = LAT::D;
+  double e_c, e_p[3], e_m[3];
+  phi_stencil<LAT, F64>(L, n, C, e_c, e_p, e_m);
+  m.I = quad_exact(L, e_c, e_p, e_m);
+  m.rho = m.M0 / m.I;
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    m.F[a] = 0.0;
-    if (a >= D) continue;
-    double fext = L.g[a];
-    if (L.has_force) fext = fext + force_at<F64>(L, a, k, dnf);
-    m.F[a] = fext + hpc * (e_p[a] - e_m[a]);
-  }
+  for (int a = 0; a < 3; ++a) m.F[a] = a < D ? force_exact<F64>(L, n, C, a, m.rho, e_p[a], e_m[a]) : 0.0;
   if (!DRAG || !L.drag_model) {
 #pragma unroll
     for (int a = 0; a < 3; ++a) m.u[a] = a < D ? __fma_rn(0.5, m.F[a], m.J[a]) / m.M0 : 0.0;

@@ -88,6 +88,7 @@ struct StepLaunch {
   // row kernel shape: consumer warps and input stages per block (0 = the
   // compiled default; the planner writes back what it chose)
   int row_consumers, row_stages;
+  int exact_split;  // FP64: plain steps share the operations of a cell between four warps
 };
 
 // Launch of a step that follows another step of the same chain (k > 0 of a

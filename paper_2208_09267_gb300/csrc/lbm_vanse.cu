@@ -1187,7 +1187,7 @@ extern "C" int lbm_vanse_launch_shape(lbm_vanse_t h, int *shape) {
   if (!h || !shape) return fail(h, LBM_EINVAL, "NULL argument");
   shape[0] = h->ls.row ? 2 : (h->p.storage == LBM_FP64 ? 0 : 1);
   shape[1] = h->ls.row ? h->ls.row_consumers : (int)h->ls.block.x;
-  shape[2] = h->ls.row ? h->ls.row_stages : (int)h->ls.block.y;
+  shape[2] = h->ls.row ? h->ls.row_stages : (h->ls.exact_split ? 4 : (int)h->ls.block.y);
   shape[3] = h->ls.row ? h->ls.row_grid : (int)(h->ls.grid.x * h->ls.grid.y * h->ls.grid.z);
   return LBM_OK;
 }

@@ -21,6 +21,9 @@ pytestmark = pytest.mark.gpu
     ("D3Q19", (47, 53, 67), 2, (0, 0)),       # 128 threads a block, a part-filled last one
     ("D3Q27", (13, 7, 5), 6, (0, 0)),
     ("D3Q27", (13, 7, 5), 0, (96, 1)),
+    ("D2Q9", (64, 152, 1), 3, (0, 0)),        # the largest lattice whose cells four warps share
+    ("D2Q9", (64, 153, 1), 0, (0, 0)),        # and the next
+    ("D3Q27", (21, 20, 23), 2, (0, 0)),
 ])
 def test_fp64_step_at_block_edges_is_bit_identical(lattice, shape, walls, block):
     N = int(np.prod(shape))
@@ -33,6 +36,6 @@ def test_fp64_step_at_block_edges_is_bit_identical(lattice, shape, walls, block)
     gpu.set_force(g, force)
     gpu.init_equilibrium()
     P = oracle.Problem(lattice, *shape, tau=0.7, walls=walls, eps_ref=eps, g=g, force=force)
-    gpu.step(6)
+    gpu.step(6, check_every=-1)
     f = P.run(P.init(), 0, 6)
     assert np.array_equal(gpu.populations(), f)
