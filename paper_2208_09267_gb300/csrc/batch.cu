@@ -33,7 +33,9 @@ LatticeDev *handle_device_desc(lbm_vanse_t h);
 const LatticeDev &handle_mirror(lbm_vanse_t h);
 LatticeDev &handle_mirror_mut(lbm_vanse_t h);
 int handle_push(lbm_vanse_t h);
-int handle_push_changed(lbm_vanse_t h, LatticeDev *last, int *pushed);
+int handle_push_changed(lbm_vanse_t h, int *pushed);
+void handle_replay_begin(lbm_vanse_t h);
+void handle_replay_end(lbm_vanse_t h, long long s);
 cudaStream_t handle_stream(lbm_vanse_t h);
 void set_global_error(const char *msg);
 int sm_count();
@@ -210,7 +212,6 @@ struct HostMember {
   long long budget;
   int type;
   int row_class;  // batched row kernel class, or -1 (one-cell-per-thread tiles)
-  LatticeDev pushed;  // the descriptor as the device holds it (valid after the first push)
   int group;      // parity of the member's time when the row tables were built
   int nrows;      // work items of the batched row kernel (tiles of up to 8 fluid rows)
   long long last_check_n;
@@ -587,7 +588,7 @@ extern "C" int lbm_vanse_batch_step(lbm_vanse_batch_t b, int k, int check) {
     LatticeDev &m = handle_mirror_mut(hm.h);
     m.have_prev = hm.have_prev ? 1 : 0;
     int pushed = 0;
-    if ((rc = handle_push_changed(hm.h, &hm.pushed, &pushed))) return bfail(rc, "member descriptor upload failed");
+    if ((rc = handle_push_changed(hm.h, &pushed))) return bfail(rc, "member descriptor upload failed");
     if (pushed || handle_stream(hm.h) != b->stream) cudaStreamSynchronize(handle_stream(hm.h));
     if (hm.row_class >= 0) {
       // members of one class are split by the parity of their time
@@ -604,6 +605,7 @@ extern "C" int lbm_vanse_batch_step(lbm_vanse_batch_t b, int k, int check) {
   if ((rc = upload_tables(b))) return rc;
   cudaGraphExec_t ge;
   if ((rc = batch_graph(b, lanes, k, check ? 1 : 0, &ge))) return rc;
+  for (auto &hm : b->members) handle_replay_begin(hm.h);
   cudaError_t e = cudaGraphLaunch(ge, b->stream);
   if (e != cudaSuccess) return bfail(LBM_ECUDA, cudaGetErrorString(e));
   count_launches((long long)k * (long long)std::count(lanes.begin(), lanes.end(), '1') + 1 + (check ? 1 : 0));
@@ -624,14 +626,9 @@ extern "C" int lbm_vanse_batch_step(lbm_vanse_batch_t b, int k, int check) {
   for (size_t i = 0; i < b->members.size(); ++i) {
     HostMember &hm = b->members[i];
     const long long s = hm.budget < k ? hm.budget : k;
+    const long long n_check = handle_mirror(hm.h).n + s - 1;
+    handle_replay_end(hm.h, s);
     if (s <= 0) continue;
-    LatticeDev &m = handle_mirror_mut(hm.h);
-    const long long n_check = m.n + s - 1;
-    m.n += s;
-    m.sig_rd = m.sig_wr;
-    // the device's copy moved the same way (advance kernel)
-    hm.pushed.n += s;
-    hm.pushed.sig_rd = hm.pushed.sig_wr;
     hm.budget -= s;
     if (check) {
       memcpy(hm.stats, b->out_host + i * kRedWidth, sizeof(hm.stats));

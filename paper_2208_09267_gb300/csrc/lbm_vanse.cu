@@ -34,6 +34,8 @@ struct lbm_vanse {
   lbm_vanse_params p;
   LatticeDev h;             // host mirror of the device descriptor
   LatticeDev *d = nullptr;  // device descriptor
+  LatticeDev pushed;        // what the device descriptor holds (it advances with the steps)
+  bool pushed_valid = false;
   cudaStream_t stream = nullptr;
   int Q = 0, D = 0;
   long long N = 0;        // cells, nx*ny*nz (the caller's dense layout)
@@ -216,10 +218,35 @@ static void sync_mirror_ptrs(lbm_vanse_t h) {
   h->h.status = h->status;
 }
 
+// Upload the descriptor where the device does not hold these values already
+// (a step, a check or a read-back after nothing but steps: a copy of 368
+// bytes each, and its wait in the stream, saved).
 static int push_mirror(lbm_vanse_t h) {
   sync_mirror_ptrs(h);
+  if (h->pushed_valid && memcmp(&h->h, &h->pushed, sizeof(LatticeDev)) == 0) return LBM_OK;
+  h->pushed_valid = false;
   CUDA_TRY(h, cudaMemcpyAsync(h->d, &h->h, sizeof(LatticeDev), cudaMemcpyHostToDevice, h->stream));
+  h->pushed = h->h;
+  h->pushed_valid = true;
   return LBM_OK;
+}
+
+// Before steps are enqueued: what the device holds is unknown until they all
+// are (a call that fails half way uploads the descriptor the next time).
+static bool forget_pushed(lbm_vanse_t h) {
+  const bool known = h->pushed_valid;
+  h->pushed_valid = false;
+  return known;
+}
+
+// k steps are enqueued: the mirror and the record of the device's copy move
+// as the advance kernel moves the descriptor.
+static void mirror_advance(lbm_vanse_t h, long long k, bool known) {
+  h->pushed_valid = known;
+  h->h.n += k;
+  h->h.sig_rd = h->h.sig_wr;
+  h->pushed.n += k;
+  h->pushed.sig_rd = h->pushed.sig_wr;
 }
 
 static void free_graphs(lbm_vanse_t h) {
@@ -790,12 +817,15 @@ extern "C" int lbm_vanse_init_equilibrium_f64(lbm_vanse_t h, const double *p0, c
 // Launch `k` plain steps (no check) starting at the mirror's time, then
 // advance the device time counter.  k == 0 is a no-op.
 static int run_plain_steps(lbm_vanse_t h, int k) {
-  for (int j = 0; j < k; ++j)
+  if (k <= 0) return LBM_OK;
+  const bool known = forget_pushed(h);
+  for (int j = 0; j < k; ++j) {
     CUDA_TRY(h, lbm::launch_step(h->h, h->d, h->h.n, j, 0, h->ls, h->stream));
-  if (k > 0) CUDA_TRY(h, lbm::launch_advance(h->d, k, h->stream));
-  if (k > 0) lbm::count_launches(k + 1);
-  h->h.n += k;
-  h->h.sig_rd = h->h.sig_wr;
+    h->h.sig_rd = h->h.sig_wr;  // a pending shift change was the first step's
+  }
+  CUDA_TRY(h, lbm::launch_advance(h->d, k, h->stream));
+  lbm::count_launches(k + 1);
+  mirror_advance(h, k, known);
   return LBM_OK;
 }
 
@@ -838,18 +868,23 @@ static int get_graph(lbm_vanse_t h, int parity, int steps, cudaGraphExec_t *out)
 static int run_steps(lbm_vanse_t h, long long k) {
   int rc;
   if (k <= 0) return LBM_OK;
-  // a pending shift change or an odd start is handled by single steps
-  if (h->h.sig_rd != h->h.sig_wr || (h->h.n & 1)) {
+  // a pending shift change or an odd start is handled outside the graphs: as
+  // one chain where no graph follows (the one-cell kernel reads the pending
+  // change from the descriptor, so it takes it as a step of its own)
+  const bool pending = h->h.sig_rd != h->h.sig_wr;
+  if (pending || (h->h.n & 1)) {
     if ((rc = push_mirror(h))) return rc;
-    if ((rc = run_plain_steps(h, 1))) return rc;
-    --k;
+    const int first = k < kGraphChunk && (!pending || h->ls.row || h->p.storage == LBM_FP64) ? (int)k : 1;
+    if ((rc = run_plain_steps(h, first))) return rc;
+    k -= first;
   }
   while (k >= kGraphChunk) {
     cudaGraphExec_t ge;
     if ((rc = get_graph(h, 0, kGraphChunk, &ge))) return rc;
+    const bool known = forget_pushed(h);
     CUDA_TRY(h, cudaGraphLaunch(ge, h->stream));
     lbm::count_launches(kGraphChunk + 1);
-    h->h.n += kGraphChunk;
+    mirror_advance(h, kGraphChunk, known);
     k -= kGraphChunk;
   }
   if (k > 0 && (rc = run_plain_steps(h, (int)k))) return rc;
@@ -861,6 +896,7 @@ static int run_steps(lbm_vanse_t h, long long k) {
 static int run_check_step(lbm_vanse_t h) {
   int rc;
   if ((rc = push_mirror(h))) return rc;
+  const bool known = forget_pushed(h);
   CUDA_TRY(h, lbm::launch_step(h->h, h->d, h->h.n, 0, 1, h->ls, h->stream));
   CUDA_TRY(h, lbm::launch_advance(h->d, 1, h->stream));
   CUDA_TRY(h, lbm::launch_finalize(h->partials, h->nblocks, h->stats_dev, h->stream));
@@ -869,8 +905,7 @@ static int run_check_step(lbm_vanse_t h) {
                               cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(h, cudaMemcpyAsync(h->stats_host + 32, h->status, sizeof(int), cudaMemcpyDeviceToHost,
                               h->stream));
-  h->h.sig_rd = h->h.sig_wr;
-  h->h.n += 1;
+  mirror_advance(h, 1, known);
   return LBM_OK;
 }
 
@@ -1158,17 +1193,17 @@ LatticeDev *handle_device_desc(lbm_vanse_t h) { return h->d; }
 const LatticeDev &handle_mirror(lbm_vanse_t h) { return h->h; }
 LatticeDev &handle_mirror_mut(lbm_vanse_t h) { return h->h; }
 int handle_push(lbm_vanse_t h) { return push_mirror(h); }
-// Upload the descriptor only if it differs from *last (what the device was
-// last given); *pushed tells whether it did.
-int handle_push_changed(lbm_vanse_t h, LatticeDev *last, int *pushed) {
+// Upload the descriptor if the device does not hold it; *pushed tells whether.
+int handle_push_changed(lbm_vanse_t h, int *pushed) {
   sync_mirror_ptrs(h);
-  *pushed = 0;
-  if (memcmp(&h->h, last, sizeof(LatticeDev)) == 0) return LBM_OK;
-  int rc;
-  if ((rc = push_mirror(h))) return rc;
-  *last = h->h;
-  *pushed = 1;
-  return LBM_OK;
+  *pushed = !(h->pushed_valid && memcmp(&h->h, &h->pushed, sizeof(LatticeDev)) == 0);
+  return push_mirror(h);
+}
+// A batch replay is about to be launched / has run s steps of this member.
+void handle_replay_begin(lbm_vanse_t h) { forget_pushed(h); }
+void handle_replay_end(lbm_vanse_t h, long long s) {
+  if (s > 0) mirror_advance(h, s, true);
+  h->pushed_valid = true;
 }
 cudaStream_t handle_stream(lbm_vanse_t h) { return h->stream; }
 void set_global_error(const char *msg) { g_last_error = msg; }
