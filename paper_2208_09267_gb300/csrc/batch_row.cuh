@@ -223,7 +223,9 @@ __global__ void __launch_bounds__(BatchRowCfg<LAT, ST, P>::kThreads, MINB)
       issued_upto = j;
       __syncwarp();
     }
-    if (abort_flag && lane == 0) {
+    if (lane == 0) {
+      // drain: wait (full limit) for every stage whose copies may be in flight
+      // (consumers may give up after this point, too)
       for (int jj = issued_upto - NSTAGE + 1; jj <= issued_upto; ++jj)
         if (jj >= 0) mbar_wait_bounded(&full[jj % NSTAGE], (unsigned)((jj / NSTAGE) & 1));
     }

@@ -9,10 +9,11 @@
 // * One block per SM: 16 consumer warps, two producers, two storers (96
 //   registers a thread; each half of them with its own stages).  A tile
 //   belongs to one group of PITCH/64 consumer warps (tile j to group j mod
-//   NG), each warp updating 64 consecutive stored cells of it, two per lane.  A warp then waits for, and releases, only the
-//   tiles it works on: with every warp dealt chunks of every tile, a quarter
-//   of all instructions went into waiting for tiles.  The 64 cells run on over
-//   the rows of a tile, so short rows leave no lanes idle.
+//   NG), each warp updating 64 consecutive stored cells of it, two per lane.
+//   A warp then waits for, and releases, only the tiles it works on: with
+//   every warp dealt chunks of every tile, a quarter of all instructions went
+//   into waiting for tiles.  The 64 cells run on over the rows of a tile, so
+//   short rows leave no lanes idle.
 // * The results overwrite the staged populations.  In the AA pattern a cell
 //   writes exactly the slots it reads (f*_i goes where f_opp(i) came from), so
 //   a staged block, once updated, is stored back to the rows it was loaded
@@ -185,8 +186,9 @@ __global__ void __launch_bounds__(kGroupThreads, 1)
       }
     }
     if (producer) {
-      if (abort_flag && lane == 0 && !withhold) {
-        // drain: wait (full limit) for every stage whose copies may be in flight
+      if (lane == 0 && !withhold) {
+        // drain: wait (full limit) for every stage whose copies may be in
+        // flight (consumers may give up after this point, too)
         for (int jj = j - kGroupHelpers; jj >= 0 && jj >= j - NSTAGE; jj -= kGroupHelpers)
           mbar_wait_bounded(&full[jj % NSTAGE], (unsigned)((jj / NSTAGE) & 1));
       }

@@ -23,6 +23,12 @@
 // the number of copies per cell: the producer warp's copy issue, not DRAM,
 // bounds rows of a few dozen cells staged one by one.
 //
+// The kernel below is the FP32 one: consumers deal the tiles' chunks among
+// themselves and store straight to global memory, and DRAM bounds it (256^3
+// D3Q19 424 us a step, 0.93 of the measured copy bandwidth).  FP16 lattices
+// take the stage layout, the copies and the per-cell update from here and run
+// them in consumer groups (step_group.cuh).
+//
 // Requirements (checked by the host before choosing this kernel): rows
 // stored at a pitch nxp that is a multiple of 8 elements (so every copy
 // starts and ends on a 16-byte boundary), nxp <= PITCH <= 512, fewer than
@@ -58,8 +64,8 @@ constexpr int row_consumers() {
 constexpr int kRowProducers = LBM_ROW_PRODUCERS;
 template <int MINB>
 constexpr int row_consumers_single() { return row_consumers<MINB>() - (kRowProducers - 1); }
-// FP16 plain steps of D2Q9/D3Q19 update two adjacent cells per lane
-// (update_row_pair); D3Q27's larger state would spill
+// batched FP16 plain steps of D2Q9/D3Q19 update two adjacent cells per lane
+// (update_row_pair); D3Q27's larger state would spill there
 template <class LAT, class ST>
 constexpr bool row_pair_lattice() { return sizeof(ST) == 2 && LAT::Q <= 19; }
 constexpr unsigned kWaitSpins = 1u << 22;  // bounded mbarrier wait
@@ -1131,9 +1137,9 @@ __global__ void __launch_bounds__((row_consumers_single<MINB>() + kRowProducers)
       }
       __syncwarp();
     }
-    if (abort_flag && lane == 0) {
+    if (lane == 0) {
       // drain: wait (full limit) for every stage whose copies this warp may
-      // still have in flight
+      // still have in flight (consumers may give up after this point, too)
       for (int jj = issued_upto; jj >= 0 && jj > issued_upto - NSTAGE * kRowProducers; jj -= kRowProducers)
         mbar_wait_bounded(&full[jj % NSTAGE], (unsigned)((jj / NSTAGE) & 1));
     }

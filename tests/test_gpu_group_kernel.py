@@ -70,3 +70,21 @@ def test_the_step_after_a_refresh_equals_its_check_step(lattice, shape, walls):
         out.append(lat.populations())
         lat.close()
     assert np.array_equal(*out)
+
+
+@pytest.mark.parametrize("lattice,shape", [("D3Q19", (128, 64, 64)), ("D3Q27", (40, 24, 20))])
+def test_wait_limit_ends_the_fp16_step(lattice, shape):
+    """With the copies withheld (nothing is in flight) every wait of the groups,
+    producers and storers runs out: the step reports the timeout and the handle
+    keeps working with the normal limit."""
+    lat = lbm.Lattice(lattice, shape, tau=0.6, storage="fp16", kernel="row")
+    lat.set_force((1e-6, 0, 0))
+    lat.set_wait_limit(64, withhold_copies=True)
+    with pytest.raises(lbm.LbmError) as e:
+        lat.step(2)
+    assert e.value.code == -5
+    lat.set_wait_limit(0, withhold_copies=False)
+    lat.init_equilibrium()
+    st = lat.step(4)
+    assert not st["nan_seen"] and st["mass"] > 0
+    lat.close()
