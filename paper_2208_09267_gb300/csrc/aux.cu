@@ -67,7 +67,8 @@ StepLaunch make_launch(int nx, int ny, int nz, int bx, int by) {
 // that still gives 8 blocks per SM, else one warp per block.  64 x 64 cells
 // are 128 warps, one SM each: 10.0 us a step (18.7 as 16 blocks of 256
 // threads, 10.8 as 32 of 128); 256 x 256: 32.6 us (35.9 in blocks of 128 or
-// more); 48^3 and 64^3 do not depend on it.
+// more); 48^3 and 64^3 do not depend on it.  (One set of warps to a cell;
+// plain steps of lattices this small run step_exact_split_kernel.)
 StepLaunch make_launch_exact(int nx, int ny, int nz, int bx, int by) {
   StepLaunch ls = make_launch(nx, ny, nz, bx, by);
   const long long cells = (long long)nx * ny * nz;

@@ -115,7 +115,7 @@ __device__ __forceinline__ double force_at(const LatticeDev &L, int a, long long
 // sign exactly, (4.5 cu) cu and (9 cu) cF do not).  About 240 operations per
 // D2Q9 cell, 430 D3Q19, 600 D3Q27: a 48^3 D3Q27 step 138 us (before 240), a
 // 64 x 64 D2Q9 step 9.6 us (26, most of it from the smaller blocks of
-// make_launch_exact).
+// make_launch_exact; 6.1 with four warps to 32 cells, step_exact.cu).
 
 // sum over the velocities of one set of c_ia v_a, terms in ascending a
 template <class LAT>

@@ -112,9 +112,6 @@ inline cudaError_t launch_chained(void (*fn)(P...), dim3 grid, dim3 block, size_
   c.dynamicSmemBytes = smem;
   c.stream = s;
   c.attrs = &attr;
-#ifdef LBM_NO_PDL
-  chained = false;
-#endif
   c.numAttrs = chained ? 1 : 0;
   return cudaLaunchKernelEx(&c, fn, static_cast<P>(args)...);
 }
