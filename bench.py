@@ -81,14 +81,18 @@ def kernel_source_hash() -> str:
     """Hash of the D3Q19 row kernel's sources with comments and blank space
     removed: a profile stays valid across comment edits, not code edits."""
     h = hashlib.sha256()
-    for name in ("step_row.cuh", "step_row_pair.cuh", "step_fast.cuh", "step_fast_d3q19.cu", "lattice.cuh",
-                 "internal.h"):
+    for name in ("step_row.cuh", "step_row_pair.cuh", "step_group.cuh", "step_fast.cuh", "step_row_d3q19_f32.cu",
+                 "step_row_d3q19_f16.cu", "lattice.cuh", "internal.h"):
         with open(os.path.join(ROOT, "paper_2208_09267_gb300", "csrc", name)) as fh:
             text = fh.read()
         text = re.sub(r"/\*.*?\*/", " ", text, flags=re.S)
         text = re.sub(r"//[^\n]*", " ", text)
         h.update(" ".join(text.split()).encode())
     return h.hexdigest()[:16]
+
+
+def row_kernel_name(storage: str) -> str:
+    return "step_group_kernel" if storage == "fp16" else "step_row_kernel"
 
 
 class ClockSampler:
@@ -318,7 +322,7 @@ def run_gpu(args, rank, world):
         st = lat.step(1)  # one check step (not timed) to confirm the run is sane
         if st["nan_seen"]:
             raise RuntimeError(f"{storage}: NaN after the timed steps")
-        kname = "step_row_kernel" if lat.row_kernel else "step_fast_kernel"
+        kname = row_kernel_name(storage) if lat.row_kernel else "step_fast_kernel"
         results[storage] = {"total_ms": total_ms, "kernel_ms": step_ms / nk, "launches": launches,
                             "clocks": clk.summary(), "mass": st["mass"],
                             "kernel": f"{kname}<D3Q19,{'float' if storage == 'fp32' else '__half'}>",
@@ -440,7 +444,7 @@ def run_porous(steps=200, warmup=10, shape=(512, 256, 256), storages=("fp32", "f
         out[storage] = {"glups": cells / (ms * 1e-3) / 1e9, "ms_per_step": ms, "bytes_per_cell": bpc,
                         "achieved_gbs": bpc * cells / (ms * 1e-3) / 1e9,
                         "frac": bpc * cells / (ms * 1e-3) / 1e9 / peak,
-                        "kernel": "step_row_kernel" if lat.row_kernel else "step_fast_kernel",
+                        "kernel": row_kernel_name(storage) if lat.row_kernel else "step_fast_kernel",
                         "nan_seen": bool(st["nan_seen"]), "clocks": clk.summary()}
         lat.close()
     return out
