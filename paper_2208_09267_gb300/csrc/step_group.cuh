@@ -23,8 +23,8 @@
 // 256^3 D3Q19 with d_t phi: 287 us a step, 58.5 GLUPS, 0.72 of the measured
 // copy bandwidth (381 us as two blocks of 6 consumers and output stages);
 // 128^3: 42 us (56); D3Q27 512 x 256 x 256 with walls: 0.84 ms, 0.66 (0.98).
-// The issue slots are 61-64 % used; what bounds it now is the instructions of
-// the update (738 / 1048 per 64 cells, even / odd step).  One producer and one
+// The issue slots are 65-69 % used; what bounds it now is the instructions of
+// the update (730 / 1054 per 64 cells, even / odd step).  One producer and one
 // storer: 373 us at 256^3 (the groups wait for tiles).
 #pragma once
 
