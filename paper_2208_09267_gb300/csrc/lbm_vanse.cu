@@ -36,6 +36,7 @@ struct lbm_vanse {
   LatticeDev *d = nullptr;  // device descriptor
   LatticeDev pushed;        // what the device descriptor holds (it advances with the steps)
   bool pushed_valid = false;
+  bool captured = false;  // the caller has captured calls of this handle
   cudaStream_t stream = nullptr;
   int Q = 0, D = 0;
   long long N = 0;        // cells, nx*ny*nz (the caller's dense layout)
@@ -218,16 +219,29 @@ static void sync_mirror_ptrs(lbm_vanse_t h) {
   h->h.status = h->status;
 }
 
+// Whether the caller captures the handle's stream, or has done so: what is
+// captured runs when, and as often as, the caller replays it, so what the
+// device holds is not known from the calls and every upload is made.
+static bool caller_captures(lbm_vanse_t h) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (!h->captured && (cudaStreamIsCapturing(h->stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone)) {
+    cudaGetLastError();
+    h->captured = true;
+  }
+  return h->captured;
+}
+
 // Upload the descriptor where the device does not hold these values already
 // (a step, a check or a read-back after nothing but steps: a copy of 368
 // bytes each, and its wait in the stream, saved).
 static int push_mirror(lbm_vanse_t h) {
   sync_mirror_ptrs(h);
-  if (h->pushed_valid && memcmp(&h->h, &h->pushed, sizeof(LatticeDev)) == 0) return LBM_OK;
+  const bool known = !caller_captures(h);
+  if (known && h->pushed_valid && memcmp(&h->h, &h->pushed, sizeof(LatticeDev)) == 0) return LBM_OK;
   h->pushed_valid = false;
   CUDA_TRY(h, cudaMemcpyAsync(h->d, &h->h, sizeof(LatticeDev), cudaMemcpyHostToDevice, h->stream));
   h->pushed = h->h;
-  h->pushed_valid = true;
+  h->pushed_valid = known;
   return LBM_OK;
 }
 
@@ -242,7 +256,7 @@ static bool forget_pushed(lbm_vanse_t h) {
 // k steps are enqueued: the mirror and the record of the device's copy move
 // as the advance kernel moves the descriptor.
 static void mirror_advance(lbm_vanse_t h, long long k, bool known) {
-  h->pushed_valid = known;
+  h->pushed_valid = known && !caller_captures(h);
   h->h.n += k;
   h->h.sig_rd = h->h.sig_wr;
   h->pushed.n += k;
@@ -1203,7 +1217,7 @@ int handle_push_changed(lbm_vanse_t h, int *pushed) {
 void handle_replay_begin(lbm_vanse_t h) { forget_pushed(h); }
 void handle_replay_end(lbm_vanse_t h, long long s) {
   if (s > 0) mirror_advance(h, s, true);
-  h->pushed_valid = true;
+  h->pushed_valid = !caller_captures(h);
 }
 cudaStream_t handle_stream(lbm_vanse_t h) { return h->stream; }
 void set_global_error(const char *msg) { g_last_error = msg; }
