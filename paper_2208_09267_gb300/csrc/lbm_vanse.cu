@@ -882,15 +882,18 @@ static int get_graph(lbm_vanse_t h, int parity, int steps, cudaGraphExec_t *out)
 static int run_steps(lbm_vanse_t h, long long k) {
   int rc;
   if (k <= 0) return LBM_OK;
-  // a pending shift change or an odd start is handled outside the graphs: as
-  // one chain where no graph follows (the one-cell kernel reads the pending
-  // change from the descriptor, so it takes it as a step of its own)
+  // a pending shift change or an odd start is handled outside the graphs,
+  // whose kernels start at an even time: as many steps as lead there, or the
+  // whole call as one chain where no graph follows (the one-cell kernel reads
+  // the pending change from the descriptor, so it takes it as a step of its
+  // own)
   const bool pending = h->h.sig_rd != h->h.sig_wr;
   if (pending || (h->h.n & 1)) {
     if ((rc = push_mirror(h))) return rc;
-    const int first = k < kGraphChunk && (!pending || h->ls.row || h->p.storage == LBM_FP64) ? (int)k : 1;
-    if ((rc = run_plain_steps(h, first))) return rc;
-    k -= first;
+    const int lead = k < kGraphChunk ? (int)k : (h->h.n & 1 ? 1 : 2);
+    const int first = pending && !h->ls.row ? 1 : lead;
+    if ((rc = run_plain_steps(h, first)) || (rc = run_plain_steps(h, lead - first))) return rc;
+    k -= lead;
   }
   while (k >= kGraphChunk) {
     cudaGraphExec_t ge;
