@@ -123,22 +123,16 @@ __device__ __forceinline__ void macro_ff(const LatticeDev &L, const FieldConsts 
   for (int a = 0; a < D; ++a) m.u[a] = b[a] / den;
 }
 
-// Moments at the device-side time.  Sums run over opposite pairs: their sum
+// Moments of one cell.  Sums run over opposite pairs: their sum
 // enters M0, their difference J, by weight class (at most four).  The cell's
 // own rest state rho0 sigma(x) is left out of the sums (the weights add to
 // one, the velocities to zero) and added to M0; at even n (ODD = false) all
 // values are stored against it and the sums are over the stored values alone.
 template <class LAT, class ST, bool ODD>
-__global__ void __launch_bounds__(256) moments_ff_kernel(const LatticeDev *__restrict__ Lp, float *rho, float *p,
-                                                         float *u) {
+__device__ __forceinline__ void moments_cell_ff(const LatticeDev *__restrict__ Lp, const FieldConsts &k, int x, int y,
+                                                int z, float *rho, float *p, float *u) {
   constexpr int Q = LAT::Q, D = LAT::D;
   const LatticeDev &L = *Lp;
-  __shared__ FieldConsts k;
-  load_consts<true>(L, k);
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  const int z = blockIdx.z;
-  if (x >= L.nx || y >= L.ny) return;
   const Coords C = make_coords(x, y, z, L.nx, L.ny, L.nz, L.nxp);
   // outputs are dense: index (z*ny + y)*nx + x, N = nx*ny*nz
   const long long o = ((long long)z * L.ny + y) * L.nx + x;
@@ -202,6 +196,22 @@ __global__ void __launch_bounds__(256) moments_ff_kernel(const LatticeDev *__res
   if (p) p[o] = ((m.rho - k.rho0) * ff_of(1.0 / 3.0)).h;
   if (u)
     for (int a = 0; a < 3; ++a) u[a * N + o] = a < D ? m.u[a].h : 0.f;
+}
+
+// At the device-side time: a captured call gives the fields of its replay, so
+// the layout of the populations follows the descriptor's time, not the host's.
+template <class LAT, class ST>
+__global__ void __launch_bounds__(256) moments_ff_kernel(const LatticeDev *__restrict__ Lp, float *rho, float *p,
+                                                         float *u) {
+  const LatticeDev &L = *Lp;
+  __shared__ FieldConsts k;
+  load_consts<true>(L, k);
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  const int y = blockIdx.y * blockDim.y + threadIdx.y;
+  const int z = blockIdx.z;
+  if (x >= L.nx || y >= L.ny) return;
+  if (L.n & 1) moments_cell_ff<LAT, ST, true>(Lp, k, x, y, z, rho, p, u);
+  else moments_cell_ff<LAT, ST, false>(Lp, k, x, y, z, rho, p, u);
 }
 
 // Write f_i/w_i = v to a slot: v - rho0 sigma against the newest shift.
@@ -275,14 +285,8 @@ __global__ void __launch_bounds__(256) init_ff_kernel(const LatticeDev *__restri
 template <class LAT>
 static void moments_lat(const LatticeDev &h, const LatticeDev *L_dev, float *rho, float *p, float *u,
                         const StepLaunch &ls, cudaStream_t s) {
-  const bool odd = (h.n & 1) != 0;
-  if (h.storage == 1) {
-    if (odd) moments_ff_kernel<LAT, float, true><<<ls.grid, ls.block, 0, s>>>(L_dev, rho, p, u);
-    else moments_ff_kernel<LAT, float, false><<<ls.grid, ls.block, 0, s>>>(L_dev, rho, p, u);
-  } else {
-    if (odd) moments_ff_kernel<LAT, __half, true><<<ls.grid, ls.block, 0, s>>>(L_dev, rho, p, u);
-    else moments_ff_kernel<LAT, __half, false><<<ls.grid, ls.block, 0, s>>>(L_dev, rho, p, u);
-  }
+  if (h.storage == 1) moments_ff_kernel<LAT, float><<<ls.grid, ls.block, 0, s>>>(L_dev, rho, p, u);
+  else moments_ff_kernel<LAT, __half><<<ls.grid, ls.block, 0, s>>>(L_dev, rho, p, u);
 }
 
 cudaError_t launch_moments_ff(const LatticeDev &h, const LatticeDev *L_dev, float *rho, float *p, float *u,
