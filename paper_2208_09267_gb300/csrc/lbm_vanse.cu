@@ -222,12 +222,14 @@ static void sync_mirror_ptrs(lbm_vanse_t h) {
 // Whether the caller captures the handle's stream, or has done so: what is
 // captured runs when, and as often as, the caller replays it, so what the
 // device holds is not known from the calls and every upload is made.
-static bool caller_captures(lbm_vanse_t h) {
+static bool capturing(lbm_vanse_t h) {
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  if (!h->captured && (cudaStreamIsCapturing(h->stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone)) {
-    cudaGetLastError();
-    h->captured = true;
-  }
+  if (cudaStreamIsCapturing(h->stream, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
+}
+static bool caller_captures(lbm_vanse_t h) {
+  if (!h->captured && capturing(h)) h->captured = true;
   return h->captured;
 }
 
@@ -828,14 +830,24 @@ extern "C" int lbm_vanse_init_equilibrium_f64(lbm_vanse_t h, const double *p0, c
 
 // ---------------------------------------------------------------- stepping
 
+// The mirror as the launches of steps see it.  Steps that the caller captures
+// may be replayed on another phi: they take the stage layout that has room for
+// d_t phi, which holds a phi without one as well.
+static LatticeDev launch_view(lbm_vanse_t h) {
+  LatticeDev m = h->h;
+  if (!m.has_deps && capturing(h)) m.has_deps = 1;
+  return m;
+}
+
 // Launch `k` plain steps (no check) starting at the mirror's time, then
 // advance the device time counter.  k == 0 is a no-op.
 static int run_plain_steps(lbm_vanse_t h, int k) {
   if (k <= 0) return LBM_OK;
   const bool known = forget_pushed(h);
+  LatticeDev m = launch_view(h);
   for (int j = 0; j < k; ++j) {
-    CUDA_TRY(h, lbm::launch_step(h->h, h->d, h->h.n, j, 0, h->ls, h->stream));
-    h->h.sig_rd = h->h.sig_wr;  // a pending shift change was the first step's
+    CUDA_TRY(h, lbm::launch_step(m, h->d, m.n, j, 0, h->ls, h->stream));
+    m.sig_rd = m.sig_wr;  // a pending shift change was the first step's
   }
   CUDA_TRY(h, lbm::launch_advance(h->d, k, h->stream));
   lbm::count_launches(k + 1);
@@ -895,7 +907,15 @@ static int run_steps(lbm_vanse_t h, long long k) {
     if ((rc = run_plain_steps(h, first)) || (rc = run_plain_steps(h, lead - first))) return rc;
     k -= lead;
   }
+  // within the caller's capture single launches (no graph can be captured
+  // there, and one from before would keep its stage layout)
+  const bool plain = k >= kGraphChunk && capturing(h);
   while (k >= kGraphChunk) {
+    if (plain) {
+      if ((rc = run_plain_steps(h, kGraphChunk))) return rc;
+      k -= kGraphChunk;
+      continue;
+    }
     cudaGraphExec_t ge;
     if ((rc = get_graph(h, 0, kGraphChunk, &ge))) return rc;
     const bool known = forget_pushed(h);
@@ -914,7 +934,7 @@ static int run_check_step(lbm_vanse_t h) {
   int rc;
   if ((rc = push_mirror(h))) return rc;
   const bool known = forget_pushed(h);
-  CUDA_TRY(h, lbm::launch_step(h->h, h->d, h->h.n, 0, 1, h->ls, h->stream));
+  CUDA_TRY(h, lbm::launch_step(launch_view(h), h->d, h->h.n, 0, 1, h->ls, h->stream));
   CUDA_TRY(h, lbm::launch_advance(h->d, 1, h->stream));
   CUDA_TRY(h, lbm::launch_finalize(h->partials, h->nblocks, h->stats_dev, h->stream));
   lbm::count_launches(3);

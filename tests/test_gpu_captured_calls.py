@@ -46,3 +46,40 @@ def test_a_captured_read_back_gives_the_fields_of_its_replay(lattice, shape, wal
             assert torch.equal(got, want)
     del g
     lat.close()
+
+
+@pytest.mark.parametrize("storage", ["fp32", "fp16"])
+@pytest.mark.parametrize("steps", [2, 66])
+@pytest.mark.parametrize("lattice,shape", [("D2Q9", (40, 9, 1)), ("D3Q19", (256, 5, 4)), ("D3Q27", (64, 6, 5)),
+                                           ("D3Q27", (320, 5, 4))])
+def test_captured_steps_follow_a_phi_that_starts_to_vary(lattice, shape, steps, storage):
+    """Steps captured on a static phi replay on one with a time derivative, and
+    on a static one again (phi_ref, and with it the shift, stays the same)."""
+    import torch
+    n = int(np.prod(shape))
+    rng = np.random.default_rng(n)
+    e = (0.5 + 0.4 * rng.random(n)).astype(np.float32)
+    d = (1e-5 * rng.standard_normal(n)).astype(np.float32)
+    s = torch.cuda.Stream()
+    lats = []
+    for stream in (s.cuda_stream, None):
+        lat = lbm.Lattice(lattice, shape, tau=0.6, storage=storage, kernel="row", fp16_rounding="nearest", stream=stream)
+        lat.set_epsilon(e)
+        lat.set_force((1e-5, -2e-6, 3e-6))
+        lat.init_equilibrium()
+        lat.step(steps, check_every=-1)
+        lats.append(lat)
+    lat, ref = lats
+    g = _capture(s, lambda: lat.step(steps, check_every=-1))
+    for phi in (None, (e, d), (e, None)):
+        # the handle's time stays that of the capture's end
+        if phi:
+            lat.set_epsilon(*phi, n_ref=lat.steps_done)
+            ref.set_epsilon(*phi, n_ref=ref.steps_done)
+        with torch.cuda.stream(s):
+            g.replay()
+        ref.step(steps, check_every=-1)
+        assert np.array_equal(lat.populations(), ref.populations())
+    del g
+    lat.close()
+    ref.close()
