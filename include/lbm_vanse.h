@@ -115,7 +115,11 @@ typedef struct {
                                row-staged (tiles of whole x-rows staged in
                                shared memory by TMA bulk copies; needs
                                8 <= nx <= 512, FP32 or FP16 storage and no
-                               walls on x; LBM_EINVAL otherwise) */
+                               walls on x; LBM_EINVAL otherwise).  FP16
+                               lattices with rho0 below 2^-20 or above 2^60
+                               always step one cell per thread: the packed
+                               divisions of their row-staged kernel would
+                               leave the float range. */
   int fp16_rounding;        /* LBM_FP16_SHIFTED stores: 0 = stochastic
                                rounding (unbiased; random bits from a
                                counter-based hash of cell and step, so runs

@@ -360,11 +360,12 @@ extern "C" int lbm_vanse_batch_add(lbm_vanse_batch_t b, lbm_vanse_t h, long long
   hm.type = type_of(m.lattice, m.storage);
   hm.row_class = -1;
   // the batched row kernel takes the member unless its lattice was created
-  // for the one-cell-per-thread kernel (explicitly, or by its drag law or
-  // closure), is one-dimensional, or its rows do not fit the kernel
+  // for the one-cell-per-thread kernel (explicitly, or by its drag law,
+  // closure or FP16 density), is one-dimensional, or its rows do not fit the
+  // kernel
   lbm_vanse_params p;
   if (lbm_vanse_get_params(h, &p) == LBM_OK && p.kernel != 1 /* one cell per thread */ && !p.drag_model &&
-      !(p.les_cs > 0.0) && m.lattice != LBM_D1Q3 && m.nx >= 8 && m.nxp <= 512 && !(m.walls & 1u) &&
+      !(p.les_cs > 0.0) && (m.storage == LBM_FP32 || packed_division_range(m.rho0)) && m.lattice != LBM_D1Q3 && m.nx >= 8 && m.nxp <= 512 && !(m.walls & 1u) &&
       m.ncell <= 0x7fffffffLL) {
     const int nyf = (m.walls & 2u) ? m.ny - 2 : m.ny, nzf = (m.walls & 4u) ? m.nz - 2 : m.nz;
     const int pitch = m.nxp <= 256 ? 256 : 512;

@@ -49,7 +49,7 @@ struct LatticeDev {
   float scale, inv_scale;  // 2^k, 2^-k (FP16); 1, 1 otherwise
   // the parameters above rounded to float once on the host, so the FP32
   // kernels convert nothing per cell (double conversions run on the narrow
-  // FP64 pipe): rho0, omega, 3 cf, 9 cf, qw0, qw1, g, cf
+  // FP64 pipe): rho0, omega, 3 cf, 9 cf, qw0, qw1 (FP16: times kDivScale), g, cf
   float rho0f, omegaf, cf3f, cf9f, qw0f, qw1f, gf[3], cff;
   // reductions of a check step
   double *partials;        // per-block partial sums, kRedWidth each
@@ -75,6 +75,14 @@ struct LatticeDev {
   float les_cf;            // 18 sqrt(2) C^2
   float tau0f;
 };
+
+// Packed divisions of FP16 steps (step_row_pair.cuh).  FP16 kernels form
+// kDivScale int phi dV (the scale is in qw0f and qw1f), a normal float for
+// every phi down to the least subnormal one; lattices of a density rho0 outside
+// the range step in the one-cell-per-thread kernel, which divides with the
+// operators.
+constexpr float kDivScale = 0x1p24f;
+inline bool packed_division_range(double rho0) { return rho0 >= 0x1p-20 && rho0 <= 0x1p60; }
 
 constexpr int kRedWidth = 12;  // M0, mom x/y/z, |du|^2, |u|^2, nan, F x/y/z, spare x2
 

@@ -205,8 +205,9 @@ static void sync_mirror_ptrs(lbm_vanse_t h) {
   m.omegaf = (float)m.omega;
   m.cf3f = 3.0f * (float)m.cf;
   m.cf9f = 9.0f * (float)m.cf;
-  m.qw0f = (float)m.qw0;
-  m.qw1f = (float)m.qw1;
+  const float qscale = m.storage == LBM_FP16_SHIFTED ? lbm::kDivScale : 1.0f;
+  m.qw0f = (float)m.qw0 * qscale;
+  m.qw1f = (float)m.qw1 * qscale;
   for (int a = 0; a < 3; ++a) m.gf[a] = (float)m.g[a];
   m.cff = (float)m.cf;
   h->h.pop = h->pop;
@@ -369,7 +370,8 @@ extern "C" int lbm_vanse_create(const lbm_vanse_params *p, lbm_vanse_t *out) {
   h->nblocks = (int)(h->ls.grid.x * h->ls.grid.y * h->ls.grid.z);
   h->ls.row_consumers = p->row_consumers;
   h->ls.row_stages = p->row_stages;
-  if (p->kernel != 1 && p->storage != LBM_FP64 && !p->drag_model && !(p->les_cs > 0.0)) {
+  if (p->kernel != 1 && p->storage != LBM_FP64 && !p->drag_model && !(p->les_cs > 0.0) &&
+      (p->storage == LBM_FP32 || lbm::packed_division_range(p->rho0))) {
     const int ok = lbm::plan_row_kernel(p->lattice, p->storage, p->nx, h->nxp, p->ny, p->nz, p->walls, h->ls);
     if (!ok && p->kernel == 2) {
       delete h;

@@ -289,7 +289,8 @@ __device__ __forceinline__ void update_cell_fast(const LatticeDev &L, long long 
   if (qa & 1u) nb += e_xp + e_xm;
   if (qa & 2u) nb += e_yp + e_ym;
   if (qa & 4u) nb += e_zp + e_zm;
-  const float I = L.qw0f * e_c + L.qw1f * nb;
+  float I = L.qw0f * e_c + L.qw1f * nb;
+  if (sizeof(ST) == 2) I *= 1.0f / kDivScale;  // (the weights of FP16 lattices carry it)
   const float rho = M0 / I;
 
   // 5. eq. (pressForce) plus the external force density

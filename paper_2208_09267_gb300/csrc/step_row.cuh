@@ -759,8 +759,8 @@ __device__ __forceinline__ void update_row_chunk(const LatticeDev &L, unsigned c
   if (qa & 1u) nb += e_xp + e_xm;
   if (qa & 2u) nb += e_yp + e_ym;
   if (qa & 4u) nb += e_zp + e_zm;
-  const float I = fmaf(L.qw0f, e_c, L.qw1f * nb);
-  const float pc2 = M0 / I * (0.5f / 3.0f);  // c_s^2 rho~ / 2
+  const float I = fmaf(L.qw0f, e_c, L.qw1f * nb);  // FP16: times kDivScale
+  const float pc2 = M0 / I * (kScaled ? 0.5f / 3.0f * kDivScale : 0.5f / 3.0f);  // c_s^2 rho~ / 2
   float F0 = fmaf(pc2, e_xp - e_xm, L.gf[0]);
   float F1 = fmaf(pc2, e_yp - e_ym, L.gf[1]);
   float F2 = D == 3 ? fmaf(pc2, e_zp - e_zm, L.gf[2]) : 0.f;

@@ -39,15 +39,18 @@ __device__ __forceinline__ P2 ld_h2(const __half *p) {
 __device__ __forceinline__ P2 ld_f2(const float *p) { return *reinterpret_cast<const float2 *>(p); }
 __device__ __forceinline__ float ldh(const __half *p) { return __half2float(*p); }
 
-// 1/b and a/b of both cells, correctly rounded for normal operands (the
-// scalar update divides with the IEEE operators): Newton's iteration on the
-// hardware's approximate reciprocal, then Markstein's correction q + y (a -
-// b q) with the exact FMA remainder, applied until the remainder is that of
-// the nearest quotient (IBM J. Res. Dev. 34, 1990).  Packed for two cells it
-// takes a third of the instructions of four operator divisions and no branch.
-// Operands within 2^-100 .. 2^100 in magnitude: M0 is a sum of halves (at
-// least 2^-56 in magnitude, or zero, where u is not finite either way) and
-// int phi dV is close to the half sigma beside it.
+// 1/b and a/b of both cells, rounded as the IEEE operators of the scalar
+// update round them: Newton's iteration on the hardware's approximate
+// reciprocal, then Markstein's correction q + y (a - b q) with the exact FMA
+// remainder, applied until the remainder is that of the nearest quotient (IBM
+// J. Res. Dev. 34, 1990).  Packed for two cells it takes a third of the
+// instructions of four operator divisions and no branch.  Range: b between
+// 2^-125 and 2^100 and a between 2^-98 and 2^61 in magnitude, so that no
+// approximation is flushed and no remainder loses bits.  M0 is there, or zero
+// (u is not finite either way), for the densities of packed_division_range: it
+// is a float sum of multiples of 2^-98 (halves times 2^-24 or more times
+// weights, and differences of halves times rho0).  int phi dV comes times
+// kDivScale, a power of two that changes no rounding.
 __device__ __forceinline__ float rcp_approx(float a) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
@@ -203,10 +206,10 @@ __device__ __forceinline__ void update_row_pair(const LatticeDev &L, unsigned ch
   P2 nb = mul2(f2s(qa & 1u ? 1.f : 0.f), add2(e_xp, e_xm));
   nb = fma2(f2s(qa & 2u ? 1.f : 0.f), add2(e_yp, e_ym), nb);
   if (D == 3) nb = fma2(f2s(qa & 4u ? 1.f : 0.f), add2(e_zp, e_zm), nb);
-  const P2 I = fma2(f2s(L.qw0f), e_c, mul2(f2s(L.qw1f), nb));
-    const P2 invM = recip2(M0);
-  const P2 rho = quot2(M0, I, recip2(I));  // rho~ = M0 / int phi dV
-  const P2 pc2 = mul2(rho, f2s(0.5f / 3.0f));
+  const P2 I = fma2(f2s(L.qw0f), e_c, mul2(f2s(L.qw1f), nb));  // kDivScale int phi dV
+  const P2 invM = recip2(M0);
+  const P2 rho = quot2(M0, I, recip2(I));  // rho~ / kDivScale
+  const P2 pc2 = mul2(rho, f2s(0.5f / 3.0f * kDivScale));
   P2 F0 = fma2(pc2, sub2(e_xp, e_xm), f2s(L.gf[0]));
   P2 F1 = fma2(pc2, sub2(e_yp, e_ym), f2s(L.gf[1]));
   P2 F2 = D == 3 ? fma2(pc2, sub2(e_zp, e_zm), f2s(L.gf[2])) : f2s(0.f);
