@@ -412,6 +412,10 @@ __device__ __forceinline__ bool plain_tile(const RowCopies &c, int y0, int z, in
 // Does a tile without walls beside it wrap around in y?
 __device__ __forceinline__ bool edge_tile(const RowCopies &c, int y0, int nr) { return y0 == 0 || y0 + nr == c.ny; }
 
+// Bytes between a plane's first row and the row after its last: 64 bits, as
+// planes of 2^30 cells and more pass 2^32 bytes.
+__host__ __device__ constexpr long long plane_span(int ny, unsigned row_bytes) { return (long long)ny * row_bytes; }
+
 // Stage a plain tile: one lane issues the copies of every block in a row,
 // unrolled over compile-time directions.  With the blocks spread over the
 // lanes instead, each copy is issued on its own all the same (its operands
@@ -433,7 +437,7 @@ __device__ __forceinline__ void issue_plain_copies(const RowCopies &c, unsigned 
   const bool lo = EDGE && y0 == 0, hi = EDGE && y0 + nr == c.ny;
   // n rows from src; the first, or the last, of them wraps around
   auto run = [&](unsigned dst, const char *src, int n, unsigned row_bytes, bool first, bool last) {
-    const unsigned span = (unsigned)c.ny * row_bytes;
+    const long long span = plane_span(c.ny, row_bytes);
     if (first) {
       copy(dst, src + span, row_bytes);
       dst += row_bytes;
@@ -453,7 +457,7 @@ __device__ __forceinline__ void issue_plain_copies(const RowCopies &c, unsigned 
       if (lo || hi) run(dst, src, nr + 2, row_bytes, lo, hi);
       else copy(dst, src, (unsigned)(nr + 2) * row_bytes);
     } else {
-      const unsigned span = (unsigned)c.ny * row_bytes;
+      const long long span = plane_span(c.ny, row_bytes);
       copy(dst, lo ? src + span : src, row_bytes);
       copy(dst + slot_bytes, src + row_bytes, row_bytes);
       copy(dst + 2 * slot_bytes, hi ? src + 2 * row_bytes - span : src + 2 * row_bytes, row_bytes);
@@ -540,14 +544,14 @@ __device__ __forceinline__ void store_plain_copies(const RowCopies &c, unsigned 
     unsigned from = stage + i * Lay::kPopBytes;
     int n = nr;
     if (cy > 0 && lo) {  // the first row wraps around
-      copy(p + (unsigned)c.ny * pb, from, pb);
+      copy(p + plane_span(c.ny, pb), from, pb);
       p += pb;
       from += pb;
       --n;
     }
     if (cy < 0 && hi) {  // the last one does
       --n;
-      copy(p + (long long)n * pb - (unsigned)c.ny * pb, from + n * pb, pb);
+      copy(p + (long long)n * pb - plane_span(c.ny, pb), from + n * pb, pb);
     }
     if (n > 0) copy(p, from, (unsigned)n * pb);
     dst += c.plane_bytes;
