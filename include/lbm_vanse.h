@@ -392,6 +392,10 @@ LBM_API int lbm_vanse_batch_remove(lbm_vanse_batch_t b, lbm_vanse_t h);
    with lbm_vanse_batch_stats after the call; the call synchronises).
    A member whose budget is spent idles. */
 LBM_API int lbm_vanse_batch_step(lbm_vanse_batch_t b, int k, int check);
+/* Limitation: the batched checks keep no velocity of the previous check, so
+   out->residual is -1 after a member's first check and 0 from its second on
+   (not the change of the flow), unless the lattice was stepped alone with a
+   residual_tol before. */
 LBM_API int lbm_vanse_batch_stats(lbm_vanse_batch_t b, lbm_vanse_t h, lbm_vanse_stats *out);
 LBM_API int lbm_vanse_batch_size(lbm_vanse_batch_t b);
 

@@ -343,16 +343,6 @@ extern "C" int lbm_vanse_batch_add(lbm_vanse_batch_t b, lbm_vanse_t h, long long
   for (auto &hm : b->members)
     if (hm.h == h) return bfail(LBM_EINVAL, "lattice is already a member");
   if ((int)b->members.size() >= b->max_members) return bfail(LBM_ENOMEM, "batch member table is full");
-  // residual tracking needs the previous check's velocity
-  LatticeDev &mm = handle_mirror_mut(h);
-  if (!mm.u_prev) {
-    void *p = nullptr;
-    if (cudaMallocAsync(&p, (size_t)3 * mm.ncell * sizeof(float), handle_stream(h)) != cudaSuccess) {
-      cudaGetLastError();
-      return bfail(LBM_ENOMEM, "residual buffer allocation failed");
-    }
-    mm.u_prev = static_cast<float *>(p);
-  }
   HostMember hm;
   memset(&hm, 0, sizeof(hm));
   hm.h = h;
