@@ -222,7 +222,9 @@ static void sync_mirror_ptrs(lbm_vanse_t h) {
 
 // Whether the caller captures the handle's stream, or has done so: what is
 // captured runs when, and as often as, the caller replays it, so what the
-// device holds is not known from the calls and every upload is made.
+// device holds is not known from the calls and no upload is left out where a
+// call makes one (steps that start at an even time on an unchanged descriptor
+// make none: they go on from the device's time).
 static bool capturing(lbm_vanse_t h) {
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(h->stream, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
@@ -249,7 +251,7 @@ static int push_mirror(lbm_vanse_t h) {
 }
 
 // Before steps are enqueued: what the device holds is unknown until they all
-// are (a call that fails half way uploads the descriptor the next time).
+// are (after a call that failed half way the next one uploads the descriptor).
 static bool forget_pushed(lbm_vanse_t h) {
   const bool known = h->pushed_valid;
   h->pushed_valid = false;
@@ -896,6 +898,7 @@ static int get_graph(lbm_vanse_t h, int parity, int steps, cudaGraphExec_t *out)
 static int run_steps(lbm_vanse_t h, long long k) {
   int rc;
   if (k <= 0) return LBM_OK;
+  if (!h->pushed_valid && !caller_captures(h) && (rc = push_mirror(h))) return rc;
   // a pending shift change or an odd start is handled outside the graphs,
   // whose kernels start at an even time: as many steps as lead there, or the
   // whole call as one chain where no graph follows (the one-cell kernel reads
