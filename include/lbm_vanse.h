@@ -161,7 +161,9 @@ typedef struct {
   int row_stages;           /* row-staged kernel: rows staged in flight per
                                block (0 = default; 2 .. compiled maximum).
                                Neither changes the arithmetic, only the
-                               launch shape; the autotuner picks them. */
+                               launch shape; the autotuner picks them.  FP16
+                               lattices have one shape and take neither
+                               (values in range are accepted). */
 } lbm_vanse_params;
 
 /* Global sums of the state at time n (pre-collision), taken on a check step
@@ -350,8 +352,9 @@ LBM_API int lbm_vanse_uses_row_kernel(lbm_vanse_t h);
 /* Launch shape of the handle's step (not in the paper; what the autotuner
    and the benchmark record): shape[0] = kernel (0 FP64 one cell per
    thread, 1 FP32/FP16 one cell per thread, 2 row-staged), then for the
-   row-staged kernel consumer warps, staged rows and grid blocks, for the
-   others block x, block y and grid blocks.  shape: 4 ints, caller-owned. */
+   row-staged kernel consumer warps, staged rows (with a d_t phi; more may fit
+   without) and grid blocks, for the others block x, block y and grid blocks.
+   shape: 4 ints, caller-owned. */
 LBM_API int lbm_vanse_launch_shape(lbm_vanse_t h, int *shape);
 
 /* Time counter n and lattice description. */

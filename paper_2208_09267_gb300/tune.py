@@ -92,7 +92,8 @@ def tune_step(lattice="D3Q19", storage="fp32", shape=(128, 128, 128), tau=0.6, s
     rows) when the lattice qualifies, and the one-cell-per-thread kernel
     with each block shape, on a lattice of this size.  Caches and returns
     (best, timings): best = {"kernel": 1|2, "block": [bx, by], "row_shape":
-    [consumers, stages] or None}, timings in ms per step per candidate."""
+    [consumers, stages] or None}, timings in ms per step per candidate.  FP16
+    lattices have one row shape, tried once."""
     import torch
     cache = cache or Cache()
     key = "step/" + bucket_key(lattice, storage, shape)
@@ -123,7 +124,7 @@ def tune_step(lattice="D3Q19", storage="fp32", shape=(128, 128, 128), tau=0.6, s
             configs[name] = cfg
         lat.close()
     if storage != "fp64":
-        for rs in row_shapes or ROW_SHAPES:
+        for rs in [(0, 0)] if storage == "fp16" else row_shapes or ROW_SHAPES:
             trial(2, (0, 0), rs)
     for bx, by in blocks or BLOCK_CANDIDATES:
         if by > ny or bx > 2 * max(nx, 32):
