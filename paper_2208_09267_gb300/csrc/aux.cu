@@ -68,15 +68,17 @@ StepLaunch make_launch(int nx, int ny, int nz, int bx, int by) {
 // are 128 warps, one SM each: 10.0 us a step (18.7 as 16 blocks of 256
 // threads, 10.8 as 32 of 128); 256 x 256: 32.6 us (35.9 in blocks of 128 or
 // more); 48^3 and 64^3 do not depend on it.  (One set of warps to a cell;
-// plain steps of lattices this small run step_exact_split_kernel.)
+// plain steps of up to two warps per SM run step_exact_split_kernel: us a step
+// with the split and without, D2Q9 of 9604 cells 8.7 and 9.7, of 10816 cells
+// 11.0 and 9.6; D3Q27 of 9261 17.2 and 22.9, of 10648 29.1 and 23.0.)
 StepLaunch make_launch_exact(int nx, int ny, int nz, int bx, int by) {
   StepLaunch ls = make_launch(nx, ny, nz, bx, by);
   const long long cells = (long long)nx * ny * nz;
   if (bx <= 0 || by <= 0) {
     int t = 256;
-    while (t > 32 && (cells + t - 1) / t < 8LL * 152) t /= 2;
+    while (t > 32 && (cells + t - 1) / t < 8LL * kChipSMs) t /= 2;
     ls.block = dim3(t, 1, 1);
-    ls.exact_split = t == 32 && cells <= 304LL * 32;  // see step_exact_split_kernel
+    ls.exact_split = t == 32 && cells <= 2LL * kChipSMs * 32;
   }
   ls.block_threads = (int)(ls.block.x * ls.block.y);
   ls.grid = dim3((unsigned)((cells + ls.block_threads - 1) / ls.block_threads), 1, 1);
@@ -195,7 +197,7 @@ cudaError_t launch_shift(const LatticeDev &h, const float *eps, __half *sig, cud
   // ones (each row of a walk waits for its loads: a walk of 32 rows takes 17
   // to 20 us, on a 64^2 lattice too)
   int seg = kShiftSeg;
-  while (seg > 2 && (long long)h.nxp * h.nz * ((h.ny + seg - 1) / seg) < 152LL * 2048) seg /= 2;
+  while (seg > 2 && (long long)h.nxp * h.nz * ((h.ny + seg - 1) / seg) < 2048LL * kChipSMs) seg /= 2;
   const long long work = (long long)h.nz * ((h.ny + seg - 1) / seg);
   const dim3 grid((unsigned)((h.nxp + block - 1) / block), (unsigned)(work < 65535 ? work : 65535));
   shift_kernel<<<grid, block, 0, s>>>(eps, sig, h.nx, h.nxp, h.ny, h.nz, h.quad_axes, (float)h.qw0,

@@ -5,10 +5,12 @@
 // SM): 465 FP64 operations per D3Q27 cell took 27 ms on 512 x 256 x 256 cells,
 // where the memory traffic takes under a millisecond.  The stored values are floats or
 // halves, so a pair of floats holds every intermediate to 48 bits, enough
-// that the single-precision results round as the FP64 ones do.  Now 2.2 ms on
-// those cells (half of the measured copy bandwidth; FP32 arithmetic bounds
-// it), 1.3 ms on D3Q19 256^3 FP16; an FP32 initial state from rest 3.3 ms on
-// the same D3Q27 cells (before 29).  Moments in double precision (rho, p, u as
+// that the single-precision results round as the FP64 ones do (values that
+// cancel, p and u near zero, to about 1e-14 absolute).  Now 2.2 ms on those
+// cells at an even time (half of the measured copy bandwidth; FP32 arithmetic
+// bounds it) and 7.6 ms at an odd one, where every value carries its slot's
+// shift; 0.96 and 2.9 ms on D3Q19 256^3 FP16.  An FP32 initial state from rest
+// takes 3.3 ms on the same D3Q27 cells (before 29).  Moments in double precision (rho, p, u as
 // double) keep the FP64 kernel.
 #include "exact.cuh"
 #include "ff.cuh"
@@ -34,7 +36,6 @@ struct FieldConsts {
   ff rho0, qw0, qw1, g[3], drag_lin, drag_q, dn, dnf;
 };
 
-template <bool DRAG>
 __device__ __forceinline__ void load_consts(const LatticeDev &L, FieldConsts &k) {
   if (threadIdx.x == 0 && threadIdx.y == 0) {
     k.rho0 = ff_of(L.rho0);
@@ -43,7 +44,7 @@ __device__ __forceinline__ void load_consts(const LatticeDev &L, FieldConsts &k)
     for (int a = 0; a < 3; ++a) k.g[a] = ff_of(L.g[a]);
     k.dn = ff_of((double)(L.n - L.n_eps));
     k.dnf = ff_of((double)(L.n - L.n_force));
-    if (DRAG && L.drag_model) {
+    if (L.drag_model) {
       k.drag_lin = ff_of(L.drag_c1 * ((L.tau0 - 0.5) / 3.0) / (L.drag_d * L.drag_d));
       k.drag_q = ff_of(L.drag_c2 / L.drag_d);
     }
@@ -205,7 +206,7 @@ __global__ void __launch_bounds__(256) moments_ff_kernel(const LatticeDev *__res
                                                          float *u) {
   const LatticeDev &L = *Lp;
   __shared__ FieldConsts k;
-  load_consts<true>(L, k);
+  load_consts(L, k);
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z;
@@ -227,7 +228,7 @@ __global__ void __launch_bounds__(256) init_ff_kernel(const LatticeDev *__restri
   constexpr int Q = LAT::Q, D = LAT::D;
   const LatticeDev &L = *Lp;
   __shared__ FieldConsts k;
-  load_consts<true>(L, k);
+  load_consts(L, k);
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z;

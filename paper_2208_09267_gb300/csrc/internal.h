@@ -86,6 +86,8 @@ inline bool packed_division_range(double rho0) { return rho0 >= 0x1p-20 && rho0 
 
 constexpr int kRedWidth = 12;  // M0, mom x/y/z, |du|^2, |u|^2, nan, F x/y/z, spare x2
 
+constexpr int kChipSMs = 152;  // GB300 (sizes of launches and tables that are also computed without a GPU)
+
 struct StepLaunch {
   dim3 grid, block;
   int block_threads;

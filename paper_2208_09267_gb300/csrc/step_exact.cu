@@ -1,5 +1,5 @@
-// step_exact.cu -- FP64 step in the canonical evaluation order, the FP64
-// FP64 and FP16 initialisation, and the moment and population kernels in FP64
+// step_exact.cu -- FP64 step in the canonical evaluation order, the FP64 and
+// FP16 initialisation, and the moment and population kernels in FP64
 // arithmetic (single-precision moments, FP32 initial state: fields_ff.cu).
 //
 // This translation unit is compiled with -fmad=false: no multiply-add is
@@ -169,8 +169,8 @@ __global__ void __launch_bounds__(256) step_exact_kernel(const LatticeDev *__res
 // which all form, warp a takes F_a and u_a; then the opposite pairs are dealt
 // to the warps.  About 95 operations deep for D2Q9; the same operations on
 // every value, so the same bits.  Worth it while the chip is not full: up to
-// two such warps a quarter (9728 cells).  64 x 64 D2Q9: 6.1 us a step
-// (9.0 with one warp for 32 cells).
+// two such blocks an SM, 9728 cells (make_launch_exact).  64 x 64 D2Q9: 6.1 us
+// a step (9.0 with one warp for 32 cells).
 constexpr int kSplit = 4;
 
 template <class LAT, bool ODD>

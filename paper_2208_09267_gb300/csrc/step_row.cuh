@@ -998,14 +998,13 @@ struct Ring {
 // Warp-specialised row kernel.  Warps kConsumerWarps .. + kRowProducers - 1
 // are the producers (one by default; producer p takes the block's tiles j =
 // p, p + P, ...): a producer stages tile j into stage j % NSTAGE once the
-// consumers have released the
-// tile that used it before (empty barrier), writes the tile's row contexts
-// and arms the full barrier with the byte count of the copies.  Each
-// producer lane owns up to two blocks of the tile's copies, set up once per
-// launch, so staging a tile costs a few instructions per lane per row
-// besides the copies.  The consumer warps wait on the full barrier, update
-// their chunks of the tile's rows and release the stage, one arrival per
-// warp.
+// consumers have released the tile that used it before (empty barrier), writes
+// the tile's row contexts, arms the full barrier with the byte count of the
+// copies and lets one lane issue them (issue_plain_tile).  The copies of tiles
+// beside a wall, and of one-row tiles that wrap around in y, are spread over
+// the lanes instead: each owns up to two blocks, set up once per launch.  The
+// consumer warps wait on the full barrier, update their chunks of the tile's
+// rows and release the stage, one arrival per warp.
 // No block-wide barrier is taken inside the loop.
 // TUNED = false: row_consumers_single() consumer warps and RowCfg's input
 // stages (kNS; kNSS when the launch asks for the static-phi layout),
@@ -1317,11 +1316,10 @@ int plan_row_t(int nx, int nxp, int ny, int nz, unsigned walls, StepLaunch &ls) 
   const bool w = (walls & 6u) != 0, p512 = nxp > 256;
   // rows of at most half the pitch are staged several at a time
   const int R = p512 ? 1 : tile_rows(256, nxp);
-  // FP32 rows narrower than the pitch also take the tiled layout with
-  // one-row tiles (halo blocks merged into one copy: 28 instead of 38 copies
-  // per row; measured +11 % at 192^3, +9 % at 224^3); FP16, whose consumers
-  // bound it, keeps the compile-time offsets
-  const bool tl = R > 1 || (sizeof(ST) == 4 && !p512 && nxp < 256);
+  // rows narrower than the pitch also take the tiled layout with one-row
+  // tiles (halo blocks merged into one copy: 28 instead of 38 copies per row;
+  // measured +11 % at 192^3, +9 % at 224^3)
+  const bool tl = R > 1 || (!p512 && nxp < 256);
   int occ = 0, ok, nc = ls.row_consumers, ns = ls.row_stages;
   if (p512)
     ok = w ? configure_row_v<LAT, ST, true, 512, (MINB > 1 ? MINB - 1 : 1), false>(occ, nc, ns)
