@@ -688,7 +688,7 @@ __device__ __forceinline__ void update_row_chunk(const LatticeDev &L, unsigned c
   const float e_own = EPS_AT(0, 0, x);
   const float sig_own = SIG_AT(0, 0, x);  // sigma_wr of this cell
   // the cell's frame: its own shift as stored (sigma_rd)
-  const float s_x = rho0 * (reshift ? __half2float(srd[cell]) : sig_own);
+  const float s_x = __fmul_rn(rho0, reshift ? __half2float(srd[cell]) : sig_own);
 
   // 1. decode: d_i = f_i/w_i - s_x (in storage units).  A value stored in
   //    another cell m carries that cell's shift: add delta_i = rho0 sigma(m)
@@ -784,9 +784,9 @@ __device__ __forceinline__ void update_row_chunk(const LatticeDev &L, unsigned c
     F2 += a2;
   }
   const float invM = 1.0f / M0;
-  const float u0 = fmaf(0.5f, F0, j0) * invM;
-  const float u1 = fmaf(0.5f, F1, j1) * invM;
-  const float u2 = D == 3 ? fmaf(0.5f, F2, j2) * invM : 0.f;
+  const float u0 = __fmul_rn(fmaf(0.5f, F0, j0), invM);
+  const float u1 = __fmul_rn(fmaf(0.5f, F1, j1), invM);
+  const float u2 = D == 3 ? __fmul_rn(fmaf(0.5f, F2, j2), invM) : 0.f;
   const float usq = fmaf(u0, u0, fmaf(u1, u1, u2 * u2));
   const float uF = fmaf(u0, F0, fmaf(u1, F1, u2 * F2));
 
@@ -883,8 +883,10 @@ __device__ __forceinline__ void update_row_chunk(const LatticeDev &L, unsigned c
       const float deqa = fmaf(M0, fmaf(cu, fmaf(4.5f, cu, 3.0f), m15usq), dM);
       const float deqb = fmaf(M0, fmaf(cu, fmaf(4.5f, cu, -3.0f), m15usq), dM);
       // Guo term / w of the pair: cf (9 cu cF - 3 u.F) +- 3 cf cF
-      // (every sum written as an explicit FMA: the rounding is then the same
-      // in every instantiation of this code, single-lattice and batched)
+      // (sums with a product are written as explicit FMAs, and products that
+      // enter plain sums, the shift and the velocities, with __fmul_rn: the
+      // rounding is then the same in every instantiation of this code,
+      // single-lattice and batched)
       const float sA = fmaf(cf9 * cu, cF, m3uF_s);
       const float sa = fmaf(cf3, cF, sA), sb = fmaf(-cf3, cF, sA);
       ENCODE_POP(i, d[i] + fmaf(omega, deqa - d[i], sa), pa_, va_);
