@@ -93,7 +93,9 @@ def tune_step(lattice="D3Q19", storage="fp32", shape=(128, 128, 128), tau=0.6, s
     with each block shape, on a lattice of this size.  Caches and returns
     (best, timings): best = {"kernel": 1|2, "block": [bx, by], "row_shape":
     [consumers, stages] or None}, timings in ms per step per candidate.  FP16
-    lattices have one row shape, tried once."""
+    lattices have one row shape, tried once; FP64 lattices also try the library's
+    default (block [0, 0], "default"): small ones then step in a kernel of their
+    own that no block shape selects."""
     import torch
     cache = cache or Cache()
     key = "step/" + bucket_key(lattice, storage, shape)
@@ -115,8 +117,8 @@ def tune_step(lattice="D3Q19", storage="fp32", shape=(128, 128, 128), tau=0.6, s
             name = f"row{ls['consumers']}x{ls['stages']}"
             cfg = {"kernel": 2, "block": [0, 0], "row_shape": [ls["consumers"], ls["stages"]]}
         else:
-            name = f"cell{ls['block'][0]}x{ls['block'][1]}"
-            cfg = {"kernel": 1, "block": list(ls["block"]), "row_shape": None}
+            name = f"cell{block[0]}x{block[1]}" if block != (0, 0) else "default"
+            cfg = {"kernel": 1, "block": list(block), "row_shape": None}
         if name not in timings:
             lat.set_force((1e-6, 0, 0))
             lat.init_equilibrium()
@@ -126,6 +128,8 @@ def tune_step(lattice="D3Q19", storage="fp32", shape=(128, 128, 128), tau=0.6, s
     if storage != "fp64":
         for rs in [(0, 0)] if storage == "fp16" else row_shapes or ROW_SHAPES:
             trial(2, (0, 0), rs)
+    else:
+        trial(1, (0, 0), None)
     for bx, by in blocks or BLOCK_CANDIDATES:
         if by > ny or bx > 2 * max(nx, 32):
             continue
